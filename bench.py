@@ -173,9 +173,8 @@ def paper_baseline(args):
             "source": "Table tab:perf_comp, D2Q9 on 4000^2"}
 
 
-TILED_KERNEL_SOURCES = ("tau1_tiled.cu", "tau1_tiled_tma.cu", "tau1_rowpair.cu", "rowpair.cuh", "tile_column.cuh",
-                        "tma.cuh", "tau1_node.cuh", "pack2.cuh", "common.cuh", "lattice.cuh", "static_for.cuh",
-                        "kernels.h")
+TILED_KERNEL_SOURCES = ("tau1_strip.cu", "strip.cuh", "moments.cuh", "mbarrier.cuh", "pack2.cuh", "common.cuh",
+                        "lattice.cuh", "static_for.cuh", "kernels.h")
 
 
 def kernel_source_hash() -> str:

@@ -71,9 +71,8 @@ typedef enum { LBM_F64 = 0, LBM_F32 = 1, LBM_F16S = 2, LBM_BF16S = 3 } lbm_stora
  * sparse layout is for the Tau1 scheme, boxes of fewer than 2^31 nodes; its
  * FP32 and FP64 results equal the dense kernels' bits. */
 /* COMPACT: the dense records, with each step's work split by tile column
- * (32 x H x 24 or 32 nodes: the tile column of the row-pair variant chosen
- * with lbm_tau1_set_variant, 2R variants as for the dense layout's row-pair
- * kernel, variant 0 by default): tile columns without
+ * (32 x H x 24 or 32 nodes, H = 8 or 16 by the variant chosen with
+ * lbm_tau1_set_variant, variant 0 by default): tile columns without
  * fluid are never read or written; those whose fluid fraction is at least the
  * threshold f* are stepped by the tiled kernel through a list; the fluid
  * nodes of the others are stepped one thread per node through a 4-byte list
@@ -218,12 +217,10 @@ lbm_status lbm_tau1_copy_plane(lbm_tau1* h, int32_t z, void* buf, int32_t to_han
 
 /* ---- Tile-shape autotuning (no counterpart in the paper, whose CPU kernels
  * fix the chunk shape at compile time, Section 3.2). The tiled kernel of the
- * 3D lattices comes in variants: [0, 2R) the row-pair form (R tile shapes:
- * warps per block, resident blocks per SM; [0, R) step 24 z planes per block,
- * [R, 2R) 32), used when nx is a multiple of 32 and ny of the tile height,
- * else the pair-position form of the same chunk height; [2R, 2R + 2T) the
- * pair-position form (T shapes, same chunk rule), TMA-staged when its tiles
- * are full. All variants give the same bits. The default is variant 0. */
+ * 3D lattices comes in variants: variant v takes strip shape v % R (R shapes:
+ * rows per strip, resident blocks per SM) and z chunks by v / R (0: chosen so
+ * that the strips fill whole waves of the GPU; 1: 32 planes, 2: 16, 3: 48).
+ * All variants give the same bits. The default is variant 0. */
 
 /* Number of variants of the handle's step kernel (1 if it has none). */
 int32_t lbm_tau1_variant_count(const lbm_tau1* h);
@@ -238,7 +235,7 @@ lbm_status lbm_tau1_set_variant(lbm_tau1* h, int32_t variant);
  * and returns its index in *chosen and its time per step in *ms_per_step
  * (either may be NULL). The trial launches rewrite only the scratch copy, so
  * the state and step counter are unchanged. Synchronises the stream.
- * Compact layout: times every pair of a row-pair variant and a threshold f*
+ * Compact layout: times every pair of a variant and a threshold f*
  * of LBM_TAU1_COMPACT_THRESHOLDS (rebuilding the lists for each), keeps the
  * fastest pair and returns the threshold's index in that list (the variant
  * is in lbm_tau1_get_compact_info); the cache is not used (the best pair
@@ -268,7 +265,7 @@ lbm_status lbm_tau1_selftest_timeout(lbm_tau1* h);
 /* Compact layout (LBM_COMPACT): how set_geometry split the box. */
 typedef struct lbm_tau1_compact_info {
     double threshold;        /* f*: fluid fraction from which a tile column is tiled */
-    int32_t variant;         /* row-pair variant of the tiled kernel (lbm_tau1_set_variant) */
+    int32_t variant;         /* variant of the tile columns (lbm_tau1_set_variant) */
     int32_t tile[3];         /* tile column: 32, H, z chunk (24 or 32, or nz if smaller) */
     int32_t tiled_ok;        /* 1 if the tiled kernel can take tile columns */
     int64_t columns;         /* tile columns of the box */
@@ -314,7 +311,7 @@ typedef struct lbm_tau1_batch lbm_tau1_batch;  /* opaque, owned by the library *
 typedef struct lbm_tau1_batch_config {
     int32_t q;            /* lbm_lattice of every box */
     int32_t storage;      /* lbm_storage of every box */
-    int32_t variant;      /* tile shape, 0 <= variant < lbm_tau1_variant_count of a tiled box / 2 */
+    int32_t variant;      /* strip shape, 0 <= variant < lbm_tau1_variant_count of a tiled box / 4 */
     int32_t capacity;     /* most boxes live at once, >= 1 */
     int32_t graph_steps;  /* steps per captured graph (>= 1; 0 = 100) */
     int32_t reserved;

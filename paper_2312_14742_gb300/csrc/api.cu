@@ -47,18 +47,17 @@ struct lbm_tau1 {
     unsigned int* dtimeouts = nullptr;  // device counter of staged-copy waits that ran out
     bool compact = false;       // compact layout: dense records, work split by tile column
     double cthr = 0.3;          // compact: fluid fraction from which a tile column is tiled
-    bool c_tiled_ok = false;    // compact: the row-pair kernel takes the box's tile columns
-    CompactTiles ctile{};       // compact: tile columns of the row-pair variant h->variant
+    bool c_tiled_ok = false;    // compact: the box is whole tile columns, and the tiled kernel takes those dense enough
+    CompactTiles ctile{};       // compact: tile columns of the variant h->variant
     int ccounted = -1;          // compact: variant whose columns ccounts holds (-1: none)
-    int64_t ccap = 0;           // compact: tile columns the three arrays below can hold
+    int64_t ccap = 0;           // compact: tile columns the two arrays below can hold
     int* ccounts = nullptr;     // compact: device fluid count of every tile column
     std::vector<int> ccounts_host;
-    int* ctiles = nullptr;      // compact: tile columns of the row-pair kernel [columns]
+    int* cstrips = nullptr;     // compact: strips of the tiled kernel [cscap], n_cstrips of them
+    int64_t cscap = 0, n_cstrips = 0;
     int* clisted = nullptr;     // compact: tile columns of the node list, then their offsets [2 columns]
     int* cnodes = nullptr;      // compact: the node list [fluid nodes]
     int64_t n_ctiles = 0, n_clisted = 0, n_cnodes = 0, c_tiled_fluid = 0, c_empty = 0;
-    cudaStream_t cside = nullptr;   // compact: the node-list kernel's stream when both kernels run
-    cudaEvent_t cfork = nullptr, cjoin = nullptr;
     int p_axis = -1;            // constant-density faces on this axis (-1: none)
     double p_lo = 1.0, p_hi = 1.0;
     std::string err;
@@ -108,12 +107,9 @@ void free_all(lbm_tau1* h)
     if (h->rescale_scratch) cudaFree(h->rescale_scratch);
     if (h->dtimeouts) cudaFree(h->dtimeouts);
     if (h->ccounts) cudaFree(h->ccounts);
-    if (h->ctiles) cudaFree(h->ctiles);
+    if (h->cstrips) cudaFree(h->cstrips);
     if (h->clisted) cudaFree(h->clisted);
     if (h->cnodes) cudaFree(h->cnodes);
-    if (h->cfork) cudaEventDestroy(h->cfork);
-    if (h->cjoin) cudaEventDestroy(h->cjoin);
-    if (h->cside) cudaStreamDestroy(h->cside);
 }
 
 // Staged-copy waits that ran out since the last call (reads the device
@@ -163,7 +159,7 @@ void fill_args(const lbm_tau1* h, StepArgs& a)
 int variant_count(const lbm_tau1* h)
 {
     if (h->cfg.q == LBM_D2Q9) return 1;
-    if (h->compact) return 2 * tau1_rowpair_shapes(h->cfg.storage);
+    if (h->compact) return 2 * tau1_tile_shapes(h->cfg.storage);
     return (!h->bgk && h->kernel == LBM_KERNEL_TILED) ? tau1_tiled_variants(h->cfg.q, h->cfg.storage) : 1;
 }
 
@@ -306,23 +302,21 @@ lbm_status build_fluid_list(lbm_tau1* h)
     return LBM_OK;
 }
 
-// Compact layout: classes the tile columns of the row-pair variant
-// h->variant by their fluid counts (counted once per geometry and variant)
+// Compact layout: classes the tile columns of variant h->variant by their fluid counts (counted once per geometry and variant)
 // with threshold h->cthr and uploads the two lists; the node list is written
 // by a kernel from the flags.
 lbm_status build_compact(lbm_tau1* h)
 {
     const lbm_tau1_config& c = h->cfg;
-    h->ctile = compact_tiles(c.q, c.storage, h->variant);
+    h->ctile = compact_tiles(c.storage, h->variant);
     const CompactTiles& ct = h->ctile;
     const int64_t nb = compact_tile_columns(ct, c.nx, c.ny, c.nz);
     if (h->ccounted != h->variant) {
         if (nb > h->ccap) {
-            for (int** p : {&h->ccounts, &h->ctiles, &h->clisted})
+            for (int** p : {&h->ccounts, &h->clisted})
                 if (*p) { cudaFree(*p); *p = nullptr; }
             h->ccap = 0;
             LBM_CUDA(h, cudaMalloc((void**)&h->ccounts, (size_t)nb * sizeof(int)), "compact: counts");
-            LBM_CUDA(h, cudaMalloc((void**)&h->ctiles, (size_t)nb * sizeof(int)), "compact: tile list");
             LBM_CUDA(h, cudaMalloc((void**)&h->clisted, (size_t)2 * nb * sizeof(int)), "compact: listed columns");
             h->ccap = nb;
         }
@@ -339,14 +333,7 @@ lbm_status build_compact(lbm_tau1* h)
             LBM_CUDA(h, cudaMalloc((void**)&h->cnodes, (size_t)(nf > 0 ? nf : 1) * sizeof(int)),
                      "compact: node list");
         }
-        StepArgs a;
-        fill_args(h, a);
-        h->c_tiled_ok = tau1_rowpair_ok(c.q, c.storage, ct.shape, a);
-        if (h->c_tiled_ok && !h->cside) {
-            LBM_CUDA(h, cudaStreamCreateWithFlags(&h->cside, cudaStreamNonBlocking), "compact: side stream");
-            LBM_CUDA(h, cudaEventCreateWithFlags(&h->cfork, cudaEventDisableTiming), "compact: event");
-            LBM_CUDA(h, cudaEventCreateWithFlags(&h->cjoin, cudaEventDisableTiming), "compact: event");
-        }
+        h->c_tiled_ok = c.nx % 32 == 0 && c.ny % ct.h == 0;  // whole tile columns only
         h->ccounted = h->variant;
     }
     std::vector<int> tiles, listed, offsets;
@@ -370,9 +357,18 @@ lbm_status build_compact(lbm_tau1* h)
     h->n_ctiles = (int64_t)tiles.size();
     h->n_clisted = (int64_t)offsets.size();
     h->n_cnodes = nodes;
-    if (!tiles.empty())
-        LBM_CUDA(h, cudaMemcpyAsync(h->ctiles, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyDefault,
-                                    h->stream), "compact: tile list copy");
+    std::vector<int> items;
+    compact_strips(ct, c.nx, c.ny, c.nz, tiles, items);
+    h->n_cstrips = (int64_t)(items.size() / STRIP_ITEM);
+    if ((int64_t)items.size() > h->cscap) {
+        if (h->cstrips) { cudaFree(h->cstrips); h->cstrips = nullptr; }
+        h->cscap = 0;
+        LBM_CUDA(h, cudaMalloc((void**)&h->cstrips, items.size() * sizeof(int)), "compact: strip list");
+        h->cscap = (int64_t)items.size();
+    }
+    if (!items.empty())
+        LBM_CUDA(h, cudaMemcpyAsync(h->cstrips, items.data(), items.size() * sizeof(int), cudaMemcpyDefault,
+                                    h->stream), "compact: strip list copy");
     if (!listed.empty())
         LBM_CUDA(h, cudaMemcpyAsync(h->clisted, listed.data(), listed.size() * sizeof(int), cudaMemcpyDefault,
                                     h->stream), "compact: listed columns copy");
@@ -396,23 +392,15 @@ cudaError_t launch_kernel(const lbm_tau1* h, int variant, const StepArgs& a)
 {
     if (h->cfg.q == LBM_D2Q9) return launch_tau1_2d(h->kernel == LBM_KERNEL_SIMPLE, h->cfg.storage, a, h->stream);
     if (h->compact) {
-        // Disjoint node sets, both read from the same copy: with both lists
-        // non-empty the node-list kernel runs on a side stream forked from
-        // and joined back into the handle's stream, so that the two kernels
-        // overlap (each fills the SMs the other's tail leaves idle).
-        const bool both = h->n_ctiles > 0 && h->n_cnodes > 0;
-        cudaStream_t ls = both ? h->cside : h->stream;
-        cudaError_t e = cudaSuccess;
-        if (both) {
-            e = cudaEventRecord(h->cfork, h->stream);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(h->cside, h->cfork, 0);
-        }
-        if (e == cudaSuccess) e = launch_tau1_list(h->cfg.q, h->cfg.storage, a, h->cnodes, h->n_cnodes, ls);
-        if (e == cudaSuccess && both) e = cudaEventRecord(h->cjoin, h->cside);
+        // Disjoint node sets, both read from the same copy: the tiled kernel may
+        // start as soon as the last blocks of the node-list kernel have (it fills
+        // the SMs that their tail leaves idle). With the list on a stream of its
+        // own it was a race which of the two got the SMs first: 211 us per step
+        // (320^3, 30% fluid) where the list did, 249 us where the tiled blocks did.
+        cudaError_t e = launch_tau1_list(h->cfg.q, h->cfg.storage, a, h->cnodes, h->n_cnodes, h->stream);
         if (e == cudaSuccess)
-            e = launch_tau1_rowpair_list(h->cfg.q, h->cfg.storage, h->ctile.shape, h->ctile.zchunk, a, h->ctiles,
-                                         (int)h->n_ctiles, h->stream);
-        if (e == cudaSuccess && both) e = cudaStreamWaitEvent(h->stream, h->cjoin, 0);
+            e = launch_tau1_tiled_list(h->cfg.q, h->cfg.storage, h->ctile.shape, h->ctile.zchunk, a, h->cstrips,
+                                       (int)h->n_cstrips, h->n_cnodes > 0, h->stream);
         return e;
     }
     if (h->sparse) return launch_tau1_sparse(h->cfg.q, h->cfg.storage, a, (int)h->nf, h->nbr, h->stream);
@@ -474,7 +462,7 @@ lbm_status time_compact(lbm_tau1* h, int trials, cudaEvent_t e0, cudaEvent_t e1,
     return LBM_OK;
 }
 
-// Compact layout: times every pair of a row-pair variant and a threshold of
+// Compact layout: times every pair of a tiled variant and a threshold of
 // LBM_TAU1_COMPACT_THRESHOLDS and keeps the fastest pair.
 lbm_status autotune_compact(lbm_tau1* h, int trials, int32_t* chosen, float* ms_per_step)
 {

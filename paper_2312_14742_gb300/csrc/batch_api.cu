@@ -37,8 +37,7 @@ struct Slot {
     uint8_t* flags = nullptr;
     uint64_t bytes = 0;
     int64_t steps = 0;
-    int ntiles = 0;  // tiles per plane
-    int tma = 0;     // stepped by the staged instance (table 1), else table 0
+    int nstrips = 0;  // strips per plane
 };
 
 uint64_t round256(uint64_t b) { return (b + 255) & ~(uint64_t)255; }
@@ -50,21 +49,15 @@ struct lbm_tau1_batch {
     cudaStream_t stream = nullptr;   // the caller's stream: all steps and table edits
     cudaStream_t side = nullptr;     // admission uploads (mask copy, flags, state init)
     cudaStream_t capture = nullptr;  // private stream for graph capture
-    cudaStream_t capture2 = nullptr; // second capture branch: the other table's chain
-    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     cudaEvent_t side_done = nullptr;
     std::vector<Slot> slots;
-    // two work tables: [0] boxes stepped by the register instance, [1] by the
-    // staged (TMA) instance; both index the same box records
-    BatchTable* dtable[2] = {};
+    BatchTable* dtable = nullptr;    // the step kernel's work table
     BatchDomain* ddom = nullptr;
-    int* dlive[2] = {};
-    int* dbegin[2] = {};
-    bool nonempty[2] = {};
-    CUtensorMap* dmaps = nullptr;  // [capacity][2]
+    int* dlive = nullptr;
+    int* dbegin = nullptr;
     Stage ring[RING];
     int ring_pos = 0;
-    int grid[2] = {}, tile_h = 0;
+    int grid = 0, rows = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     uint64_t budget = 0, used = 0;
@@ -148,108 +141,75 @@ cudaError_t stage_done(Stage* s, cudaStream_t stream)
 }
 
 // Work items of a box for a chunk height.
-int box_items(const Slot& s, int chunk) { return s.ntiles * ((s.cfg.nz + chunk - 1) / chunk); }
+int box_items(const Slot& s, int chunk) { return s.nstrips * ((s.cfg.nz + chunk - 1) / chunk); }
 
-// Rebuilds the live lists and item offsets of both tables and queues their
-// upload. A table's chunk is the tallest of 32, 16, 8 planes that still gives
-// at least two items per block of its persistent grid, else 4. A change in
-// which tables are empty drops the captured graph (it launches only the
-// non-empty ones).
+// Rebuilds the live list and item offsets and queues their upload. The chunk
+// is the one with the least (waves of items over the persistent grid's warps) x (planes
+// an item forms: two beside its own, and about as much again to start).
 lbm_status upload_table(lbm_tau1_batch* b)
 {
-    int nlive = 0;
-    for (int t = 0; t < 2; ++t) {
-        int chunk = 32;
-        for (; chunk > 4; chunk /= 2) {
-            int64_t tot = 0;
-            for (const Slot& s : b->slots)
-                if (s.live && s.tma == t) tot += box_items(s, chunk);
-            if (tot >= 2 * (int64_t)b->grid[t]) break;
+    static const int chunks[] = {64, 48, 40, 32, 28, 24, 20, 16, 12, 10, 8, 6, 5, 4, 3, 2};
+    int chunk = 32;
+    int64_t best = -1;
+    for (int c : chunks) {
+        int64_t tot = 0;
+        for (const Slot& s : b->slots)
+            if (s.live) tot += box_items(s, c);
+        const int64_t warps = 4 * (int64_t)b->grid, cost = (tot + warps - 1) / warps * (c + 4);
+        if (best < 0 || cost < best) {
+            best = cost;
+            chunk = c;
         }
-        std::vector<int> live, begin;
-        int items = 0;
-        for (int i = 0; i < (int)b->slots.size(); ++i)
-            if (b->slots[i].live && b->slots[i].tma == t) {
-                live.push_back(i);
-                begin.push_back(items);
-                items += box_items(b->slots[i], chunk);
-            }
-        const int nd = (int)live.size();
-        BatchTable hdr{};
-        hdr.nitems = items;
-        hdr.ndom = nd;
-        hdr.done = 0;
-        hdr.next = 0;
-        hdr.chunk = chunk;
-        hdr.live = b->dlive[t];
-        hdr.item_begin = b->dbegin[t];
-        hdr.dom = b->ddom;
-        hdr.maps = b->dmaps;
-        const size_t lb = (size_t)nd * sizeof(int);
-        Stage* st = nullptr;
-        BCUDA(b, stage_get(b, sizeof(hdr) + 2 * lb + 16, &st), "batch: staging buffer");
-        unsigned char* p = static_cast<unsigned char*>(st->p);
-        std::memcpy(p, &hdr, sizeof(hdr));
-        if (nd) {
-            std::memcpy(p + sizeof(hdr), live.data(), lb);
-            std::memcpy(p + sizeof(hdr) + lb, begin.data(), lb);
-            BCUDA(b, cudaMemcpyAsync(b->dlive[t], p + sizeof(hdr), lb, cudaMemcpyHostToDevice, b->stream),
-                  "batch: table copy");
-            BCUDA(b, cudaMemcpyAsync(b->dbegin[t], p + sizeof(hdr) + lb, lb, cudaMemcpyHostToDevice, b->stream),
-                  "batch: table copy");
-        }
-        BCUDA(b, cudaMemcpyAsync(b->dtable[t], p, sizeof(hdr), cudaMemcpyHostToDevice, b->stream),
-              "batch: table copy");
-        BCUDA(b, stage_done(st, b->stream), "batch: staging event");
-        if ((nd > 0) != b->nonempty[t] && b->gexec) {
-            // the graph's launches follow which tables are non-empty
-            BCUDA(b, cudaStreamSynchronize(b->stream), "batch: sync before graph rebuild");
-            cudaGraphExecDestroy(b->gexec);
-            cudaGraphDestroy(b->graph);
-            b->gexec = nullptr;
-            b->graph = nullptr;
-        }
-        b->nonempty[t] = nd > 0;
-        nlive += nd;
     }
-    b->nlive = nlive;
+    std::vector<int> live, begin;
+    int items = 0;
+    for (int i = 0; i < (int)b->slots.size(); ++i)
+        if (b->slots[i].live) {
+            live.push_back(i);
+            begin.push_back(items);
+            items += box_items(b->slots[i], chunk);
+        }
+    const int nd = (int)live.size();
+    BatchTable hdr{};
+    hdr.nitems = items;
+    hdr.ndom = nd;
+    hdr.done = 0;
+    hdr.next = 0;
+    hdr.chunk = chunk;
+    hdr.live = b->dlive;
+    hdr.item_begin = b->dbegin;
+    hdr.dom = b->ddom;
+    const size_t lb = (size_t)nd * sizeof(int);
+    Stage* st = nullptr;
+    BCUDA(b, stage_get(b, sizeof(hdr) + 2 * lb + 16, &st), "batch: staging buffer");
+    unsigned char* p = static_cast<unsigned char*>(st->p);
+    std::memcpy(p, &hdr, sizeof(hdr));
+    if (nd) {
+        std::memcpy(p + sizeof(hdr), live.data(), lb);
+        std::memcpy(p + sizeof(hdr) + lb, begin.data(), lb);
+        BCUDA(b, cudaMemcpyAsync(b->dlive, p + sizeof(hdr), lb, cudaMemcpyHostToDevice, b->stream),
+              "batch: table copy");
+        BCUDA(b, cudaMemcpyAsync(b->dbegin, p + sizeof(hdr) + lb, lb, cudaMemcpyHostToDevice, b->stream),
+              "batch: table copy");
+    }
+    BCUDA(b, cudaMemcpyAsync(b->dtable, p, sizeof(hdr), cudaMemcpyHostToDevice, b->stream), "batch: table copy");
+    BCUDA(b, stage_done(st, b->stream), "batch: staging event");
+    b->nlive = nd;
     return LBM_OK;
 }
 
-// One step of every live box: one launch per non-empty table.
-cudaError_t launch_step_tables(lbm_tau1_batch* b, cudaStream_t s)
+// One step of every live box.
+cudaError_t launch_step(lbm_tau1_batch* b, cudaStream_t s)
 {
-    for (int t = 1; t >= 0; --t)
-        if (b->nonempty[t]) {
-            cudaError_t e = launch_tau1_batch(b->cfg.q, b->cfg.storage, b->cfg.variant, t == 1, b->dtable[t],
-                                              b->grid[t], s);
-            if (e != cudaSuccess) return e;
-        }
-    return cudaSuccess;
+    return launch_tau1_batch(b->cfg.q, b->cfg.storage, b->cfg.variant, b->dtable, b->grid, s);
 }
-
-int launches_per_step(const lbm_tau1_batch* b) { return (b->nonempty[0] ? 1 : 0) + (b->nonempty[1] ? 1 : 0); }
 
 lbm_status capture_graph(lbm_tau1_batch* b)
 {
     const int k = b->cfg.graph_steps;
     BCUDA(b, cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal), "batch: begin capture");
     cudaError_t le = cudaSuccess;
-    if (b->nonempty[0] && b->nonempty[1]) {
-        // the two tables hold different boxes: two independent chains of k
-        // steps, which the GPU runs side by side (one fills the other's tails)
-        le = cudaEventRecord(b->fork_ev, b->capture);
-        if (le == cudaSuccess) le = cudaStreamWaitEvent(b->capture2, b->fork_ev, 0);
-        for (int t = 1; t >= 0; --t) {
-            cudaStream_t cs = t == 1 ? b->capture : b->capture2;
-            for (int i = 0; i < k && le == cudaSuccess; ++i)
-                le = launch_tau1_batch(b->cfg.q, b->cfg.storage, b->cfg.variant, t == 1, b->dtable[t], b->grid[t], cs);
-        }
-        if (le == cudaSuccess) le = cudaEventRecord(b->join_ev, b->capture2);
-        if (le == cudaSuccess) le = cudaStreamWaitEvent(b->capture, b->join_ev, 0);
-    } else {
-        for (int i = 0; i < k && le == cudaSuccess; ++i) le = launch_step_tables(b, b->capture);
-    }
+    for (int i = 0; i < k && le == cudaSuccess; ++i) le = launch_step(b, b->capture);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(b->capture, &g);
     if (le != cudaSuccess || ee != cudaSuccess) {
@@ -284,13 +244,10 @@ void free_batch(lbm_tau1_batch* b)
         if (s.ev) { cudaEventSynchronize(s.ev); cudaEventDestroy(s.ev); }
         if (s.p) cudaFreeHost(s.p);
     }
-    for (int t = 0; t < 2; ++t) {
-        if (b->dtable[t]) cudaFree(b->dtable[t]);
-        if (b->dlive[t]) cudaFree(b->dlive[t]);
-        if (b->dbegin[t]) cudaFree(b->dbegin[t]);
-    }
+    if (b->dtable) cudaFree(b->dtable);
+    if (b->dlive) cudaFree(b->dlive);
+    if (b->dbegin) cudaFree(b->dbegin);
     if (b->ddom) cudaFree(b->ddom);
-    if (b->dmaps) cudaFree(b->dmaps);
     if (b->red_partials) cudaFree(b->red_partials);
     if (b->red_out) cudaFree(b->red_out);
     if (b->red_host) cudaFreeHost(b->red_host);
@@ -301,9 +258,6 @@ void free_batch(lbm_tau1_batch* b)
     if (b->side_done) cudaEventDestroy(b->side_done);
     if (b->side) cudaStreamDestroy(b->side);
     if (b->capture) cudaStreamDestroy(b->capture);
-    if (b->capture2) cudaStreamDestroy(b->capture2);
-    if (b->fork_ev) cudaEventDestroy(b->fork_ev);
-    if (b->join_ev) cudaEventDestroy(b->join_ev);
 }
 
 lbm_status live_slot(lbm_tau1_batch* b, int32_t slot, const char* what)
@@ -353,21 +307,14 @@ lbm_status lbm_tau1_batch_create(const lbm_tau1_batch_config* cfg, lbm_tau1_batc
     b->stream = static_cast<cudaStream_t>(cfg->cuda_stream);
     b->slots.resize((size_t)cfg->capacity);
     const int cap = cfg->capacity;
-    cudaError_t e = batch_prepare(cfg->q, cfg->storage, cfg->variant, false, &b->grid[0], &b->tile_h);
-    if (e == cudaSuccess) e = batch_prepare(cfg->q, cfg->storage, cfg->variant, true, &b->grid[1], &b->tile_h);
+    cudaError_t e = batch_prepare(cfg->q, cfg->storage, cfg->variant, &b->grid, &b->rows);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture2, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side_done, cudaEventDisableTiming);
-    for (int t = 0; t < 2; ++t) {
-        if (e == cudaSuccess) e = cudaMalloc(&b->dtable[t], sizeof(BatchTable));
-        if (e == cudaSuccess) e = cudaMalloc(&b->dlive[t], (size_t)cap * sizeof(int));
-        if (e == cudaSuccess) e = cudaMalloc(&b->dbegin[t], (size_t)cap * sizeof(int));
-    }
+    if (e == cudaSuccess) e = cudaMalloc(&b->dtable, sizeof(BatchTable));
+    if (e == cudaSuccess) e = cudaMalloc(&b->dlive, (size_t)cap * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->dbegin, (size_t)cap * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->ddom, (size_t)cap * sizeof(BatchDomain));
-    if (e == cudaSuccess) e = cudaMalloc(&b->dmaps, (size_t)cap * 2 * sizeof(CUtensorMap));
     if (e == cudaSuccess) e = cudaMalloc(&b->red_partials, (size_t)1024 * RED_FIELDS * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&b->red_out, (size_t)cap * RED_FIELDS * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->dtimeouts, sizeof(unsigned int));
@@ -470,9 +417,7 @@ lbm_status lbm_tau1_batch_admit(lbm_tau1_batch* b, const lbm_tau1_config* cfg, c
     }
     rec.buf[0] = s.buf[0];
     rec.buf[1] = s.buf[1];
-    rec.ntx = (cfg->nx + 31) / 32;
-    const int nty = (cfg->ny + b->tile_h - 1) / b->tile_h;
-    rec.ntiles = rec.ntx * nty;
+    rec.nstrips = (int)batch_strips(cfg->nx, cfg->ny, rec.a.periodic[0], b->rows);
     rec.cur = 0;
     rec.step = 0;
     for (int c = 0; c < 2; ++c)
@@ -481,24 +426,11 @@ lbm_status lbm_tau1_batch_admit(lbm_tau1_batch* b, const lbm_tau1_config* cfg, c
             rec.scale[c][4 + f] = 1.0f / sc[f];
         }
     rec.gfloor = (float)(64.0 * gmax);
-    // staged tile columns for boxes of full tiles (16-bit rows start on 16 bytes only for even nx)
-    CUtensorMap maps[2];
-    rec.tma = cfg->nx % 32 == 0 && cfg->ny % b->tile_h == 0 &&
-              !((cfg->storage == LBM_F16S || cfg->storage == LBM_BF16S) && cfg->nx % 2 != 0);
-    for (int c = 0; c < 2 && rec.tma; ++c)
-        if (encode_state_map(cfg->storage, s.buf[c], cfg->nx, cfg->ny, cfg->nz, b->tile_h + 2, &maps[c]) !=
-            cudaSuccess)
-            rec.tma = 0;
     Stage* st = nullptr;
-    BCUDA(b, stage_get(b, sizeof(rec) + sizeof(maps), &st), "batch_admit: staging buffer");
-    std::memcpy(st->p, maps, sizeof(maps));
-    std::memcpy(static_cast<unsigned char*>(st->p) + sizeof(maps), &rec, sizeof(rec));
+    BCUDA(b, stage_get(b, sizeof(rec), &st), "batch_admit: staging buffer");
+    std::memcpy(st->p, &rec, sizeof(rec));
     BCUDA(b, cudaStreamWaitEvent(b->stream, b->side_done, 0), "batch_admit: wait");
-    if (rec.tma)
-        BCUDA(b, cudaMemcpyAsync(b->dmaps + 2 * id, st->p, sizeof(maps), cudaMemcpyHostToDevice, b->stream),
-              "batch_admit: tensor map copy");
-    BCUDA(b, cudaMemcpyAsync(b->ddom + id, static_cast<unsigned char*>(st->p) + sizeof(maps), sizeof(rec),
-                             cudaMemcpyHostToDevice, b->stream),
+    BCUDA(b, cudaMemcpyAsync(b->ddom + id, st->p, sizeof(rec), cudaMemcpyHostToDevice, b->stream),
           "batch_admit: record copy");
     BCUDA(b, stage_done(st, b->stream), "batch_admit: staging event");
 
@@ -507,8 +439,7 @@ lbm_status lbm_tau1_batch_admit(lbm_tau1_batch* b, const lbm_tau1_config* cfg, c
     s.n = n;
     s.bytes = need;
     s.steps = 0;
-    s.ntiles = rec.ntiles;
-    s.tma = rec.tma;
+    s.nstrips = rec.nstrips;
     b->used += need;
     if (lbm_status r = upload_table(b)) return r;
     *slot = id;
@@ -545,11 +476,11 @@ lbm_status lbm_tau1_batch_step(lbm_tau1_batch* b, int64_t nsteps)
         if (lbm_status st = capture_graph(b)) return st;
     for (; left >= k; left -= k) {
         BCUDA(b, cudaGraphLaunch(b->gexec, b->stream), "batch_step: graph launch");
-        b->launches += k * launches_per_step(b);
+        b->launches += k;
     }
     for (; left > 0; --left) {
-        BCUDA(b, launch_step_tables(b, b->stream), "batch_step: launch");
-        b->launches += launches_per_step(b);
+        BCUDA(b, launch_step(b, b->stream), "batch_step: launch");
+        ++b->launches;
     }
     for (Slot& s : b->slots)
         if (s.live) s.steps += nsteps;

@@ -1,6 +1,6 @@
 // Compact porous layout: the dense state records, with the work of a step
 // split by tile column (a 32 x H tile of the x-y plane, a chunk of 24 or 32
-// z planes: the unit of work of one row-pair kernel variant).
+// z planes).
 //
 // The paper's kernels skip solid chunks and treat mixed chunks through the
 // node mask (Section 3.2); its bandwidth model for porous media charges a
@@ -8,18 +8,19 @@
 // (Section 5) names indirect addressing of the fluid nodes. Here each tile
 // column is classed by its fluid count c out of m nodes:
 //   - c = 0: never visited (no record is read or written);
-//   - c >= f* m: stepped by the row-pair kernel through a list of tile
-//     columns (every node of the tile is loaded, as in the dense layout);
+//   - c >= f* m: stepped by the tiled kernel, in strips cut from the runs of
+//     such tiles (every node is loaded, as in the dense layout);
 //   - 0 < c < f* m: its fluid nodes join a node list (4-byte box indices, in
 //     z, y, x order of the tile), stepped one thread per node with the
 //     neighbours read straight from the dense records (each state copy holds
 //     one more record after the box: a solid sentinel for the sources that
 //     lie outside a non-periodic face).
-// Both kernels compute every link as the dense kernels do, and the node sets
+// Both kernels compute every node as the dense kernels do, and the node sets
 // are disjoint, so a step gives the dense step's bits.
+#include <algorithm>
+
 #include "kernels.h"
-#include "static_for.cuh"
-#include "tau1_node.cuh"
+#include "moments.cuh"
 
 namespace lbm {
 
@@ -58,70 +59,85 @@ __device__ __forceinline__ void axis_sources(uint32_t c, uint32_t n, int st, boo
     off[0] = c + 1 < n ? st : (per ? -(int)(n - 1) * st : 0);
 }
 
-// One Tau1 step of the listed (fluid) box nodes, one thread per node, the
-// neighbours' records gathered from the dense state. A source outside a
-// non-periodic face is read from the sentinel record n (drho = NaN, u = 0)
-// that follows the box in both state copies, so that every source is a plain
-// load and a wall is recognised by its NaN alone. A thread issues the loads of
-// all q - 1 sources first (FP32 and 16-bit storage; FP64 one link at a time,
-// for registers), then evaluates the links in the dense kernels' order
-// (c_z = +1, 0, -1, each in k order) with their per-link arithmetic: the
-// equilibrium of a fluid source, or the reflected own equilibrium for a wall
-// (the dense kernels add these as fma(sigma, b, v) with the other term zero;
-// here the term is selected, which gives the same value, the sign of a zero
-// term aside).
-template <int Q, int ST>
-__global__ void __launch_bounds__(256) tau1_list_kernel(StepArgs a, const int* __restrict__ nodes, int count,
-                                                        DivBy by_nx, DivBy by_nxy)
-{
-    using S = Storage<ST>;
-    using T = typename S::ctype;
-    constexpr bool PRELOAD = sizeof(T) == 4;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    const uint32_t i = (uint32_t)__ldg(nodes + t);
-    const Scales sc(a.dscale);
-    T d0, ux0, uy0, uz0;
-    S::load(a.pre, i, sc.inv, d0, ux0, uy0, uz0);
-    if (isnan(d0)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
-    const uint32_t nx = (uint32_t)a.nx, nxy = nx * (uint32_t)a.ny;
-    const uint32_t sentinel = nxy * (uint32_t)a.nz;
-    const uint32_t z = by_nxy.div(i), r = i - z * nxy, y = by_nx.div(r), x = r - y * nx;
+// One Tau1 step of the listed (fluid) box nodes, the neighbours' records
+// gathered from the dense state. A source outside a non-periodic face is read
+// from the sentinel record n (drho = NaN, u = 0) that follows the box in both
+// state copies, so that every source is a plain load and a wall is recognised by
+// its NaN alone. The sums are those of moments.cuh. One thread per node: two
+// nodes per thread in packed arithmetic take a third fewer instructions but
+// leave too few warps to hide the gathers (303 us against 256 on 9.9 M nodes).
+struct ListArgs {
+    const int* nodes;
+    int count;
+    DivBy by_nx, by_nxy;
+};
+
+// What a node's sources need: the offsets per axis, and whether they are in the box.
+struct Around {
+    uint32_t i;
     int ox[3], oy[3], oz[3];
     bool ix[3], iy[3], iz[3];
-    axis_sources(x, nx, 1, a.periodic[0], ox, ix);
-    axis_sources(y, (uint32_t)a.ny, (int)nx, a.periodic[1], oy, iy);
-    axis_sources(z, (uint32_t)a.nz, (int)nxy, a.periodic[2], oz, iz);
-
-    T rd[Q], rux[Q], ruy[Q], ruz[Q];
-    auto gather = [&](auto kc) {
-        constexpr int K = decltype(kc)::value;
+    __device__ __forceinline__ void set(const StepArgs& a, const ListArgs& l, uint32_t node)
+    {
+        i = node;
+        const uint32_t nx = (uint32_t)a.nx, nxy = nx * (uint32_t)a.ny;
+        const uint32_t z = l.by_nxy.div(i), r = i - z * nxy, y = l.by_nx.div(r), x = r - y * nx;
+        axis_sources(x, nx, 1, a.periodic[0], ox, ix);
+        axis_sources(y, (uint32_t)a.ny, (int)nx, a.periodic[1], oy, iy);
+        axis_sources(z, (uint32_t)a.nz, (int)nxy, a.periodic[2], oz, iz);
+    }
+    template <int K> __device__ __forceinline__ uint32_t source(uint32_t sentinel) const
+    {
         constexpr int X = cvel(K, 0) + 1, Y = cvel(K, 1) + 1, Z = cvel(K, 2) + 1;
-        const uint32_t s = (ix[X] && iy[Y] && iz[Z]) ? i + (uint32_t)(ox[X] + oy[Y] + oz[Z]) : sentinel;
-        S::load(a.pre, s, sc.inv, rd[K], rux[K], ruy[K], ruz[K]);
-    };
-    if constexpr (PRELOAD) static_for<1, Q>(gather);
+        return (ix[X] && iy[Y] && iz[Z]) ? i + (uint32_t)(ox[X] + oy[Y] + oz[Z]) : sentinel;
+    }
+};
 
-    const T gx = gcomp<T>(a, 0), gy = gcomp<T>(a, 1), gz = gcomp<T>(a, 2);
-    const NodeMoments<T> own = node_moments<T>(d0, ux0, uy0, uz0, gx, gy, gz);
-    NodeAcc<T, Weights<Q>::NCLASS> acc;
-    acc.S[0] = own.A;  // rest direction: p = 0
+template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> load_rec(const void* base, uint32_t i, const float* inv)
+{
+    Rec<typename Storage<ST>::ctype> r;
+    Storage<ST>::load(base, i, inv, r.d, r.ux, r.uy, r.uz);
+    return r;
+}
 
-    auto link = [&](auto kc) {
+template <int Q, int ST>
+__global__ void __launch_bounds__(256, ST == ST_F64 ? 0 : (Q == 19 ? 6 : 4)) tau1_list_kernel(StepArgs a, ListArgs l)
+{
+    using T = typename Storage<ST>::ctype;
+    asm volatile("griddepcontrol.launch_dependents;");  // the tiled kernel of this step: other nodes
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const Scales sc(a.dscale);
+    const Force<T> g(a);
+    const uint32_t sentinel = (uint32_t)a.nx * (uint32_t)a.ny * (uint32_t)a.nz;
+    auto bit = [](auto kc) {
         constexpr int K = decltype(kc)::value;
-        if constexpr (!PRELOAD) gather(kc);
-        const NodeMoments<T> m = node_moments<T>(rd[K], rux[K], ruy[K], ruz[K], gx, gy, gz);
-        const T v = feq_scaled(m.A, m.H, dir_dot<K, T>(m.Px, m.Py, m.Pz));
-        const T b = feq_scaled(own.A, own.H, -dir_dot<K, T>(own.Px, own.Py, own.Pz));
-        acc.template add<Q, K>(isnan(rd[K]) ? b : v);
+        return 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
     };
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 1) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 0) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == -1) link(kc); });
-
+    if (t >= l.count) return;
+    Around A;
+    A.set(a, l, (uint32_t)__ldg(l.nodes + t));
+    Rec<T> r[Q];
+    r[0] = load_rec<ST>(a.pre, A.i, sc.inv);
+    if (isnan(r[0].d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
+    if constexpr (sizeof(T) == 4)  // every load first (FP64: as they are used, for registers)
+        static_for<1, Q>([&](auto kc) {
+            constexpr int K = decltype(kc)::value;
+            r[K] = load_rec<ST>(a.pre, A.template source<K>(sentinel), sc.inv);
+        });
+    const Moments<T> own = moments_of_record<T>(r[0].d, r[0].ux, r[0].uy, r[0].uz, g);
+    uint32_t wall = 0;
+    T sums[4];
+    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
+        constexpr int K = decltype(kc)::value;
+        if constexpr (K == 0) return own;
+        if constexpr (sizeof(T) == 8) r[K] = load_rec<ST>(a.pre, A.template source<K>(sentinel), sc.inv);
+        if (isnan(r[K].d)) wall |= bit(kc);
+        return moments_of_record<T>(r[K].d, r[K].ux, r[K].uy, r[K].uz, g);
+    }, sums);
+    add_bounce<Q, T>(own, wall, sums);
     T d, ux, uy, uz;
-    node_finish<Q, T>(acc, d, ux, uy, uz);
-    step_store<ST>(a.post, i, d, ux, uy, uz, sc.s, a.seed);
+    node_state<Q, T>(sums, d, ux, uy, uz);
+    step_store<ST>(a.post, A.i, d, ux, uy, uz, sc.s, a.seed);
 }
 
 // The sentinel record n of a state copy: drho = NaN, u = 0.
@@ -136,8 +152,8 @@ __global__ void sentinel_kernel(void* buf, uint32_t n, const float* __restrict__
 template <int Q, int ST>
 cudaError_t launch_list_t(const StepArgs& a, const int* nodes, int count, cudaStream_t s)
 {
-    const DivBy bx = DivBy::make((uint32_t)a.nx), bxy = DivBy::make((uint32_t)a.nx * (uint32_t)a.ny);
-    tau1_list_kernel<Q, ST><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(a, nodes, count, bx, bxy);
+    const ListArgs l{nodes, count, DivBy::make((uint32_t)a.nx), DivBy::make((uint32_t)a.nx * (uint32_t)a.ny)};
+    tau1_list_kernel<Q, ST><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(a, l);
     return cudaGetLastError();
 }
 
@@ -234,13 +250,15 @@ TileGeo geo_of(const CompactTiles& t, int nx, int ny, int nz)
 
 }  // namespace
 
-CompactTiles compact_tiles(int q, int storage, int variant)
+CompactTiles compact_tiles(int storage, int variant)
 {
-    const int nr = tau1_rowpair_shapes(storage);
+    const int nr = tau1_tile_shapes(storage);
     CompactTiles t;
-    t.shape = variant % nr;
+    const int v = variant % nr;
+    t.shape = nr == 1 ? 0 : (v < 2 ? 1 : 0);
     t.zchunk = variant < nr ? 24 : 32;
-    t.h = tau1_rowpair_tile_height(q, storage, t.shape);
+    t.h = v % 2 ? 16 : 8;
+    t.rows = tau1_strip_rows(storage, t.shape);
     return t;
 }
 
@@ -261,6 +279,43 @@ int64_t compact_tile_nodes(const CompactTiles& t, int nx, int ny, int nz, int b)
     const int64_t hh = ny - y0 < g.h ? ny - y0 : g.h;
     const int64_t d = nz - z0 < g.chunk ? nz - z0 : g.chunk;
     return w * hh * d;
+}
+
+void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, std::vector<int>& items)
+{
+    const TileGeo g = geo_of(t, nx, ny, nz);
+    items.clear();
+    int lanes = 32, chunk = -1;  // of the last item
+    auto pad = [&] {
+        for (; lanes < 32; ++lanes) items.push_back(items.back() < 0 ? items.back() : ~items.back());
+        if (chunk >= 0) items.push_back(chunk);
+    };
+    for (size_t i = 0; i < tiles.size();) {
+        // a run of tiles side by side, then each of its groups of rows
+        const int tile = tiles[i] % g.ntiles, c = tiles[i] / g.ntiles, tx = tile % g.ntx;
+        size_t e = i + 1;
+        while (e < tiles.size() && tiles[e] == tiles[e - 1] + 1 && tx + (int)(e - i) < g.ntx) ++e;
+        for (int j = 0; j < t.h / t.rows; ++j) {
+            const int first = (tile / g.ntx * (t.h / t.rows) + j) * (nx + 2);  // slot of column -1
+            int x = 32 * tx;
+            const int end = std::min(nx, 32 * (tx + (int)(e - i)));
+            while (x < end) {
+                if (lanes > 29 || c != chunk) {
+                    pad();
+                    lanes = 0;
+                    chunk = c;
+                }
+                const int n = std::min(end - x, 30 - lanes);
+                items.push_back(~(first + x));
+                for (int k = 1; k <= n; ++k) items.push_back(first + x + k);
+                items.push_back(~(first + x + n + 1));
+                lanes += n + 2;
+                x += n;
+            }
+        }
+        i = e;
+    }
+    pad();
 }
 
 cudaError_t launch_compact_count(const CompactTiles& t, int nx, int ny, int nz, const uint8_t* flags, int* counts,

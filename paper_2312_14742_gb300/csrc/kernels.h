@@ -2,7 +2,7 @@
 #pragma once
 
 #include <cstdint>
-#include <cuda.h>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -11,42 +11,40 @@ namespace lbm {
 
 // Tau1 step kernels (dense layout).
 cudaError_t launch_tau1_simple(int q, int storage, const StepArgs& a, cudaStream_t s);
+// Tiled kernel (tau1_strip.cu): variant v is strip shape v % R, R =
+// tau1_tile_shapes, with z chunks that fill whole waves, of 32, 16 or 48 planes (v / R).
 cudaError_t launch_tau1_tiled(int q, int storage, int variant, const StepArgs& a, cudaStream_t s);
 bool tau1_tiled_supported(int q, int storage, int64_t n);
-int tau1_tiled_variants(int q, int storage);  // (row-pair + pair-position tile shapes) x z-chunk heights
-int tau1_tile_shapes(int storage);            // tile shapes (the batched kernel's variants)
-// Staged (TMA) form of the tiled kernel: same bits; for boxes with full tiles.
-bool tau1_tiled_tma_ok(int q, int storage, int variant, const StepArgs& a);
-cudaError_t launch_tau1_tiled_tma(int q, int storage, int variant, const StepArgs& a, cudaStream_t s);
-// Tensor map of a state copy for the staged kernels: 3D {4 nx, ny, nz} values,
-// box {4 (32 + 2 XOFF), box_rows, 1}.
-cudaError_t encode_state_map(int storage, const void* base, int nx, int ny, int nz, int box_rows, CUtensorMap* map);
-// Row-pair form (shuffle exchange within rows, shared memory across warp
-// seams): same bits; for boxes with full tiles of its shape.
-int tau1_rowpair_shapes(int storage);
-bool tau1_rowpair_ok(int q, int storage, int shape, const StepArgs& a);
-cudaError_t launch_tau1_rowpair(int q, int storage, int shape, int zchunk, const StepArgs& a, cudaStream_t s);
-// Tile height (2W) of a row-pair shape (0 if none), and the row-pair kernel of
-// a shape over a list of tile columns (indices b of the grid order: tile
-// b % ntiles, z chunk b / ntiles, ntiles = (nx / 32) (ny / tile height)).
-int tau1_rowpair_tile_height(int q, int storage, int shape);
-cudaError_t launch_tau1_rowpair_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
-                                     int count, cudaStream_t s);
+int tau1_tiled_variants(int q, int storage);
+int tau1_tile_shapes(int storage);
+// Rows of a shape's strips, and the kernel of a shape over a list of strips: per
+// strip STRIP_ITEM ints, its 32 slots (ys (nx + 2) + x + 1 for column x of the
+// ys-th group of rows; ~slot where the strip does not own the column) and its
+// chunk of zchunk planes. An owned column has its neighbours in the next lanes.
+// after_list: the last launch on s is launch_tau1_list() of the same step.
+constexpr int STRIP_ITEM = 33;
+int tau1_strip_rows(int storage, int shape);
+cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
+                                   int count, bool after_list, cudaStream_t s);
 // Self-test (selftest.cu): one warp waits, bounded, on an mbarrier phase
 // that nothing completes and counts the timeout in *timeouts.
 cudaError_t launch_selftest_timeout(unsigned int* timeouts, cudaStream_t s);
 
 // Compact porous layout (compact.cu): tile columns of 32 x h x zchunk nodes,
-// the unit of the row-pair variant (shape, zchunk) (variant v of
-// [0, 2 tau1_rowpair_shapes): shape v mod R, zchunk 24 below R, else 32),
-// numbered like that kernel's grid; fluid counts per tile column, and the
-// fluid nodes of listed tile columns in row order at the given offsets.
+// numbered chunk-major, then by rows of tiles (variant v of [0, 2R), R =
+// tau1_tile_shapes: h 8 or 16 for even or odd v, zchunk 24 below R, else 32;
+// stepped in strips of the given shape and rows); fluid counts per tile column,
+// and the fluid nodes of listed tile columns in row order at the given offsets.
 struct CompactTiles {
-    int shape, zchunk, h;
+    int shape, zchunk, h, rows;
 };
-CompactTiles compact_tiles(int q, int storage, int variant);
+CompactTiles compact_tiles(int storage, int variant);
 int64_t compact_tile_columns(const CompactTiles& t, int nx, int ny, int nz);
 int64_t compact_tile_nodes(const CompactTiles& t, int nx, int ny, int nz, int b);
+// The strips that cover the given tile columns (in grid order), as
+// launch_tau1_tiled_list takes them; the box is whole tiles (nx a multiple of 32,
+// ny of the tile height).
+void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, std::vector<int>& items);
 cudaError_t launch_compact_count(const CompactTiles& t, int nx, int ny, int nz, const uint8_t* flags, int* counts,
                                  cudaStream_t s);
 cudaError_t launch_compact_nodes(const CompactTiles& t, int nx, int ny, int nz, const uint8_t* flags, const int* tiles,

@@ -1,17 +1,13 @@
-// Tensor-memory-accelerator (TMA) loads into shared memory, completed on an
-// mbarrier, for the staged tiled kernel.
+// Shared-memory addresses and bounded mbarrier waits.
 //
-// One thread issues a tiled 3D bulk copy of a box of the state into shared
-// memory; the copy reports its bytes to an mbarrier of that buffer, and every
-// thread waits for the barrier's phase before reading the box. Waits are
-// bounded: a wait that runs past its limit returns false; the kernel then
-// counts a timeout in its caller's device counter (StepArgs::timeouts, read
-// and cleared by the host, which reports LBM_ETIMEOUT), stops issuing copies
-// and storing, so that a missing completion can never hang the GPU.
+// A wait that runs past its limit returns false; its kernel then counts a
+// timeout in its caller's device counter (StepArgs::timeouts, read and cleared
+// by the host, which reports LBM_ETIMEOUT) and returns, so that a missing
+// completion can never hang the GPU.
 #pragma once
 
 #include <cstdint>
-#include <cuda.h>
+#include <cuda_runtime.h>
 
 namespace lbm {
 
@@ -52,16 +48,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     while (clock64() - t0 < (1ll << 31))
         if (mbar_try_wait(bar, parity)) return true;
     return false;
-}
-
-// Tiled 3D copy of the box at element coordinates (c0, c1, c2) into dst
-// (128-byte aligned shared memory); completion is counted on bar.
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-        : "memory");
 }
 
 }  // namespace lbm

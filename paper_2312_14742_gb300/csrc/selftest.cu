@@ -3,7 +3,7 @@
 // same device counter as the step kernels, so that a test or a health check
 // can see a wait run out and reach the host as LBM_ETIMEOUT without any fault.
 #include "kernels.h"
-#include "tma.cuh"
+#include "mbarrier.cuh"
 
 namespace lbm {
 

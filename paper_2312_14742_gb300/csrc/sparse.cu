@@ -12,12 +12,10 @@
 //   - the step reads the own record, the index and the source record of each
 //     link, and writes the own record: 2 (d+1) s + 4 (q-1) bytes per fluid
 //     node from HBM when the source records come from cache.
-// The per-link arithmetic and its order are those of the dense kernels
-// (halfway bounce-back as fma(sigma, b, v); links c_z = +1, 0, -1, each in
-// k order), so a sparse step gives the dense step's bits (FP32 and FP64).
+// The arithmetic and its order are those of the dense kernels (moments.cuh), so
+// a sparse step gives the dense step's bits (FP32 and FP64).
 #include "kernels.h"
-#include "static_for.cuh"
-#include "tau1_node.cuh"
+#include "moments.cuh"
 
 namespace lbm {
 
@@ -128,42 +126,44 @@ __global__ void __launch_bounds__(256) table_kernel(int nf, int nx, int ny, int 
     });
 }
 
-// One Tau1 step of the fluid list: one thread per fluid node.
+// One Tau1 step of the fluid list: one thread per fluid node. D3Q19 hides the
+// latency of its gathers with warps (32 registers: 55.4 us for 1.8 M nodes, 61.2
+// with the registers the compiler would take); D3Q27 does better with more loads
+// in flight per thread (75.5 us against 94.8 at 40 registers).
+constexpr int sparse_blocks(int q, int st) { return q == 19 ? (st == ST_F64 ? 0 : 8) : (st == ST_F16S ? 4 : 0); }
 template <int Q, int ST>
-__global__ void __launch_bounds__(256) tau1_sparse_kernel(StepArgs a, int nf, const int* __restrict__ nbr)
+__global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(StepArgs a, int nf, const int* __restrict__ nbr)
 {
     using S = Storage<ST>;
     using T = typename S::ctype;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf) return;
     const Scales sc(a.dscale);
-    const T gx = gcomp<T>(a, 0), gy = gcomp<T>(a, 1), gz = gcomp<T>(a, 2);
+    const Force<T> g(a);
+    // every index first: the records' loads then wait for none but their own
+    int src[Q];
+    static_for<1, Q>([&](auto kc) {
+        constexpr int K = decltype(kc)::value;
+        src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
+    });
     T d0, ux0, uy0, uz0;
     S::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
-    const NodeMoments<T> own = node_moments<T>(d0, ux0, uy0, uz0, gx, gy, gz);
-    NodeAcc<T, Weights<Q>::NCLASS> acc;
-    acc.S[0] = own.A;
-
-    auto link = [&](auto kc) {
+    const Moments<T> own = moments_of<T>(d0, ux0, uy0, uz0, g, false);
+    uint32_t wall = 0;
+    T sums[4];
+    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
         constexpr int K = decltype(kc)::value;
-        const int j = __ldg(nbr + (int64_t)(K - 1) * nf + i);
-        T v = T(0), sigma = T(1);
-        if (j >= 0) {
-            T d, ux, uy, uz;
-            S::load(a.pre, (uint32_t)j, sc.inv, d, ux, uy, uz);
-            const NodeMoments<T> m = node_moments<T>(d, ux, uy, uz, gx, gy, gz);
-            v = feq_scaled(m.A, m.H, dir_dot<K, T>(m.Px, m.Py, m.Pz));
-            sigma = T(0);
-        }
-        const T b = feq_scaled(own.A, own.H, -dir_dot<K, T>(own.Px, own.Py, own.Pz));
-        acc.template add<Q, K>(fma(sigma, b, v));
-    };
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 1) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 0) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == -1) link(kc); });
+        if constexpr (K == 0) return own;
+        const bool w = src[K] < 0;
+        T d = T(0), ux = T(0), uy = T(0), uz = T(0);
+        if (!w) S::load(a.pre, (uint32_t)src[K], sc.inv, d, ux, uy, uz);
+        if (w) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+        return moments_of<T>(d, ux, uy, uz, g, w);
+    }, sums);
+    add_bounce<Q, T>(own, wall, sums);
 
     T d, ux, uy, uz;
-    node_finish<Q, T>(acc, d, ux, uy, uz);
+    node_state<Q, T>(sums, d, ux, uy, uz);
     step_store<ST>(a.post, (uint32_t)i, d, ux, uy, uz, sc.s, a.seed);
 }
 

@@ -1,17 +1,13 @@
 // Tau1 step, one thread per node, neighbours read straight from global memory.
 //
 // The plain form of Algorithm "Tau1" (pull, AB layout) with the halfway
-// bounce-back of Algorithm "Complete Tau1 ... halfway bounce-back": for each
-// direction k the node gathers (drho, u) of x - c_k, forms the scaled
-// equilibrium and accumulates it; a wall link takes the equilibrium of the
-// node's own previous state in direction inv(k). It serves any box shape and
-// every storage format and is the cross-check of the tiled kernel: it
-// evaluates each link with the same operations in the same order (walls as
-// fma(sigma, b, v) with sigma = 1 for a wall, 0 otherwise; links in the order
-// c_z = +1, 0, -1, each in k order), so both kernels give the same bits.
+// bounce-back of Algorithm "Complete Tau1 ... halfway bounce-back": the node
+// reads every source's record, forms its moments and takes the sums of
+// moments.cuh; wall links add the node's own equilibria. It serves any box
+// shape and every storage format and is the cross-check of the tiled kernel,
+// which evaluates the same functions in the same order: both give the same bits.
 #include "kernels.h"
-#include "static_for.cuh"
-#include "tau1_node.cuh"
+#include "moments.cuh"
 
 namespace lbm {
 
@@ -30,46 +26,30 @@ __global__ void __launch_bounds__(256) tau1_simple_kernel(StepArgs a)
     const int x = (int)(i % a.nx);
     const int y = (int)((i / a.nx) % a.ny);
     const int z = (int)(i / ((int64_t)a.nx * a.ny));
-    const T gx = gcomp<T>(a, 0), gy = gcomp<T>(a, 1), gz = gcomp<T>(a, 2);
-
-    const NodeMoments<T> own = node_moments<T>(d0, ux0, uy0, uz0, gx, gy, gz);
-    NodeAcc<T, Weights<Q>::NCLASS> acc;
-    acc.S[0] = own.A;  // rest direction: p = 0
-
-    // one link: the equilibrium arriving along c_K, or the reflected one
-    auto link = [&](auto kc) {
+    const Force<T> g(a);
+    const Moments<T> own = moments_of_record<T>(d0, ux0, uy0, uz0, g);
+    uint32_t wall = 0;
+    T sums[4];
+    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
         constexpr int K = decltype(kc)::value;
+        if constexpr (K == 0) return own;
         int sx = x - cvel(K, 0), sy = y - cvel(K, 1), sz = z - cvel(K, 2);
         bool inside = true;
         if (sx < 0 || sx >= a.nx) { if (a.periodic[0]) sx = sx < 0 ? sx + a.nx : sx - a.nx; else inside = false; }
         if (sy < 0 || sy >= a.ny) { if (a.periodic[1]) sy = sy < 0 ? sy + a.ny : sy - a.ny; else inside = false; }
         if (sz < 0 || sz >= a.nz) { if (a.periodic[2]) sz = sz < 0 ? sz + a.nz : sz - a.nz; else inside = false; }
-        T d = T(0), ux = T(0), uy = T(0), uz = T(0);
-        bool solid = true;
+        T d = T(NAN), ux = T(0), uy = T(0), uz = T(0);
         if (inside) {
             const int64_t s = (int64_t)sx + (int64_t)a.nx * ((int64_t)sy + (int64_t)a.ny * sz);
             S::load(a.pre, (uint32_t)s, sc.inv, d, ux, uy, uz);
-            solid = isnan(d);
-            if (solid) d = T(0);
         }
-        // source value; a wall source contributes 0 (its moments are zeroed)
-        NodeMoments<T> m = node_moments<T>(d, ux, uy, uz, gx, gy, gz);
-        const T keep = solid ? T(0) : T(1);
-        m.A = m.A * keep;
-        m.Px = m.Px * keep;
-        m.Py = m.Py * keep;
-        m.Pz = m.Pz * keep;
-        const T v = feq_scaled(m.A, m.H, dir_dot<K, T>(m.Px, m.Py, m.Pz));
-        // reflected population: own state in direction inv(k), p(inv k) = -p(k)
-        const T b = feq_scaled(own.A, own.H, -dir_dot<K, T>(own.Px, own.Py, own.Pz));
-        acc.template add<Q, K>(fma(solid ? T(1) : T(0), b, v));
-    };
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 1) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == 0) link(kc); });
-    static_for<1, Q>([&](auto kc) { if constexpr (cvel(decltype(kc)::value, 2) == -1) link(kc); });
+        if (isnan(d)) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+        return moments_of_record<T>(d, ux, uy, uz, g);
+    }, sums);
+    add_bounce<Q, T>(own, wall, sums);
 
     T d, ux, uy, uz;
-    node_finish<Q, T>(acc, d, ux, uy, uz);
+    node_state<Q, T>(sums, d, ux, uy, uz);
     step_store<ST>(a.post, (uint32_t)i, d, ux, uy, uz, sc.s, a.seed);
 }
 
