@@ -91,7 +91,7 @@ __device__ __forceinline__ StepArgs uniform_args(const BatchDomain& D, uint32_t 
 }
 
 template <int Q, int ST, int R, int MINB>
-__global__ void __launch_bounds__(128, MINB) tau1_batch_kernel(BatchTable* T)
+__global__ void __launch_bounds__(Cfg<Q, ST, R>::NT, 4 * MINB / Cfg<Q, ST, R>::W) tau1_batch_kernel(BatchTable* T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int last;
@@ -100,10 +100,10 @@ __global__ void __launch_bounds__(128, MINB) tau1_batch_kernel(BatchTable* T)
     constexpr bool AMAX = ST == ST_F16S;
     const int nitems = uniform(T->nitems), ndom = uniform(T->ndom), chunk = uniform(T->chunk);
     const int* __restrict__ begin = T->item_begin;
-    const int warp = uniform((int)(threadIdx.x >> 5)), nwarps = 4 * (int)gridDim.x;
+    const int warp = uniform((int)(threadIdx.x >> 5)), nwarps = Cfg<Q, ST, R>::W * (int)gridDim.x;
     // each warp takes its first item by its index, then the next free one
     // (items differ in size: partial strips, partial chunks, several boxes)
-    for (int it = 4 * (int)blockIdx.x + warp; it < nitems;) {
+    for (int it = Cfg<Q, ST, R>::W * (int)blockIdx.x + warp; it < nitems;) {
         // box of this item: the last d with begin[d] <= it
         int lo = 0, hi = ndom - 1;
         while (lo < hi) {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(128, MINB) tau1_batch_kernel(BatchTable* T)
 
 template <int Q, int ST, int V>
 struct BatchKernel {
-    using Sh = ColShape<Q, typename Storage<ST>::ctype, V>;
+    using Sh = StripShape<typename Storage<ST>::ctype, V>;
     using C = Cfg<Q, ST, Sh::R>;
     static_assert(C::SMEM <= 227 * 1024, "shared memory of one block");
     static constexpr auto fn() { return tau1_batch_kernel<Q, ST, Sh::R, Sh::MINB>; }
@@ -176,6 +176,9 @@ struct BatchKernel {
     }
 };
 
+// Shape of variant 0; the others name one.
+constexpr int BATCH_SHAPE = 1;
+
 template <int Q, int ST>
 cudaError_t dispatch_v(int variant, bool prep, BatchTable* T, int& grid, int& rows, cudaStream_t s)
 {
@@ -187,10 +190,10 @@ cudaError_t dispatch_v(int variant, bool prep, BatchTable* T, int& grid, int& ro
         return variant == 0 ? go(BatchKernel<Q, ST, 0>{}) : cudaErrorInvalidValue;
     } else {
         switch (variant) {
-        case 0: return go(BatchKernel<Q, ST, dense_shape(0)>{});
-        case 1: return go(BatchKernel<Q, ST, dense_shape(1)>{});
-        case 2: return go(BatchKernel<Q, ST, dense_shape(2)>{});
-        case 3: return go(BatchKernel<Q, ST, dense_shape(3)>{});
+        case 0: return go(BatchKernel<Q, ST, BATCH_SHAPE>{});
+        case 1: return go(BatchKernel<Q, ST, 0>{});
+        case 2: return go(BatchKernel<Q, ST, 1>{});
+        case 3: return go(BatchKernel<Q, ST, 2>{});
         default: return cudaErrorInvalidValue;
         }
     }

@@ -155,7 +155,7 @@ lbm_status upload_table(lbm_tau1_batch* b)
         int64_t tot = 0;
         for (const Slot& s : b->slots)
             if (s.live) tot += box_items(s, c);
-        const int64_t warps = 4 * (int64_t)b->grid, cost = (tot + warps - 1) / warps * (c + 4);
+        const int64_t warps = STRIP_WARPS * (int64_t)b->grid, cost = (tot + warps - 1) / warps * (c + 4);
         if (best < 0 || cost < best) {
             best = cost;
             chunk = c;

@@ -66,18 +66,26 @@ __device__ __forceinline__ void axis_sources(uint32_t c, uint32_t n, int st, boo
 // its NaN alone. The sums are those of moments.cuh. One thread per node: two
 // nodes per thread in packed arithmetic take a third fewer instructions but
 // leave too few warps to hide the gathers (303 us against 256 on 9.9 M nodes).
+// Away from the faces, where all nodes of a warp are as a rule, the sources lie at
+// fixed distances: a third of the instructions went into finding them. 9.9 M
+// nodes in D3Q19 take 204 us (221 without that case, 238 link by link), in D3Q27
+// 345 (359, 342); the default split of the same box (320^3, 30% fluid) 199 us
+// and 258, where the link-by-link kernels took 225 and 351.
 struct ListArgs {
     const int* nodes;
     int count;
     DivBy by_nx, by_nxy;
 };
 
+constexpr int LIST_THREADS = 128;
+
 // What a node's sources need: the offsets per axis, and whether they are in the box.
 struct Around {
     uint32_t i;
     int ox[3], oy[3], oz[3];
     bool ix[3], iy[3], iz[3];
-    __device__ __forceinline__ void set(const StepArgs& a, const ListArgs& l, uint32_t node)
+    // true where no source lies on another side of the box
+    __device__ __forceinline__ bool set(const StepArgs& a, const ListArgs& l, uint32_t node)
     {
         i = node;
         const uint32_t nx = (uint32_t)a.nx, nxy = nx * (uint32_t)a.ny;
@@ -85,6 +93,7 @@ struct Around {
         axis_sources(x, nx, 1, a.periodic[0], ox, ix);
         axis_sources(y, (uint32_t)a.ny, (int)nx, a.periodic[1], oy, iy);
         axis_sources(z, (uint32_t)a.nz, (int)nxy, a.periodic[2], oz, iz);
+        return x - 1u < nx - 2u && y - 1u < (uint32_t)a.ny - 2u && z - 1u < (uint32_t)a.nz - 2u && nx > 2 && a.ny > 2 && a.nz > 2;
     }
     template <int K> __device__ __forceinline__ uint32_t source(uint32_t sentinel) const
     {
@@ -93,21 +102,14 @@ struct Around {
     }
 };
 
-template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> load_rec(const void* base, uint32_t i, const float* inv)
-{
-    Rec<typename Storage<ST>::ctype> r;
-    Storage<ST>::load(base, i, inv, r.d, r.ux, r.uy, r.uz);
-    return r;
-}
-
 template <int Q, int ST>
-__global__ void __launch_bounds__(256, ST == ST_F64 ? 0 : (Q == 19 ? 6 : 4)) tau1_list_kernel(StepArgs a, ListArgs l)
+__global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12 : 8)) tau1_list_kernel(StepArgs a, ListArgs l)
 {
     using T = typename Storage<ST>::ctype;
     asm volatile("griddepcontrol.launch_dependents;");  // the tiled kernel of this step: other nodes
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const Scales sc(a.dscale);
-    const Force<T> g(a);
+    const Terms<ST> terms(a, sc);
     const uint32_t sentinel = (uint32_t)a.nx * (uint32_t)a.ny * (uint32_t)a.nz;
     auto bit = [](auto kc) {
         constexpr int K = decltype(kc)::value;
@@ -115,29 +117,38 @@ __global__ void __launch_bounds__(256, ST == ST_F64 ? 0 : (Q == 19 ? 6 : 4)) tau
     };
     if (t >= l.count) return;
     Around A;
-    A.set(a, l, (uint32_t)__ldg(l.nodes + t));
-    Rec<T> r[Q];
-    r[0] = load_rec<ST>(a.pre, A.i, sc.inv);
-    if (isnan(r[0].d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
-    if constexpr (sizeof(T) == 4)  // every load first (FP64: as they are used, for registers)
-        static_for<1, Q>([&](auto kc) {
+    const bool inner = A.set(a, l, (uint32_t)__ldg(l.nodes + t));
+    const Rec<T> own_record = record<ST>(a.pre, A.i);
+    if (isnan(own_record.d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
+    auto step = [&](auto source) {
+        Rec<T> r[Q];
+        if constexpr (sizeof(T) == 4 && Q == 19)  // every load first (else as they are used, for registers)
+            static_for<1, Q>([&](auto kc) { r[decltype(kc)::value] = record<ST>(a.pre, source(kc)); });
+        const Moments<T> own = moments_of_record<ST>(own_record, terms);
+        uint32_t wall = 0;
+        T sums[4];
+        gather_sums<Q, ST>(terms, own, [&](auto kc, bool& solid) {
             constexpr int K = decltype(kc)::value;
-            r[K] = load_rec<ST>(a.pre, A.template source<K>(sentinel), sc.inv);
+            if constexpr (sizeof(T) == 8 || Q == 27) r[K] = record<ST>(a.pre, source(kc));
+            solid = isnan(r[K].d);
+            if (solid) wall |= bit(kc);
+            return r[K];
+        }, sums);
+        add_bounce<Q, T>(own, wall, sums);
+        T d, ux, uy, uz;
+        node_state<Q, T>(sums, d, ux, uy, uz);
+        step_store<ST>(a.post, A.i, d, ux, uy, uz, sc.s, a.seed);
+    };
+    // away from the faces the sources are at fixed distances
+    if (__all_sync(__activemask(), inner)) {
+        const uint32_t nx = (uint32_t)a.nx, nxy = nx * (uint32_t)a.ny;
+        step([&](auto kc) {
+            constexpr int K = decltype(kc)::value;
+            return A.i - ((uint32_t)cvel(K, 0) + (uint32_t)cvel(K, 1) * nx + (uint32_t)cvel(K, 2) * nxy);
         });
-    const Moments<T> own = moments_of_record<T>(r[0].d, r[0].ux, r[0].uy, r[0].uz, g);
-    uint32_t wall = 0;
-    T sums[4];
-    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
-        constexpr int K = decltype(kc)::value;
-        if constexpr (K == 0) return own;
-        if constexpr (sizeof(T) == 8) r[K] = load_rec<ST>(a.pre, A.template source<K>(sentinel), sc.inv);
-        if (isnan(r[K].d)) wall |= bit(kc);
-        return moments_of_record<T>(r[K].d, r[K].ux, r[K].uy, r[K].uz, g);
-    }, sums);
-    add_bounce<Q, T>(own, wall, sums);
-    T d, ux, uy, uz;
-    node_state<Q, T>(sums, d, ux, uy, uz);
-    step_store<ST>(a.post, A.i, d, ux, uy, uz, sc.s, a.seed);
+    } else {
+        step([&](auto kc) { return A.template source<decltype(kc)::value>(sentinel); });
+    }
 }
 
 // The sentinel record n of a state copy: drho = NaN, u = 0.
@@ -153,7 +164,7 @@ template <int Q, int ST>
 cudaError_t launch_list_t(const StepArgs& a, const int* nodes, int count, cudaStream_t s)
 {
     const ListArgs l{nodes, count, DivBy::make((uint32_t)a.nx), DivBy::make((uint32_t)a.nx * (uint32_t)a.ny)};
-    tau1_list_kernel<Q, ST><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(a, l);
+    tau1_list_kernel<Q, ST><<<(unsigned)((count + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0, s>>>(a, l);
     return cudaGetLastError();
 }
 
@@ -255,7 +266,9 @@ CompactTiles compact_tiles(int storage, int variant)
     const int nr = tau1_tile_shapes(storage);
     CompactTiles t;
     const int v = variant % nr;
-    t.shape = nr == 1 ? 0 : (v < 2 ? 1 : 0);
+    // four rows per strip, but two in the 16-bit formats (by default) and for v 2, 3
+    const bool sixteen = storage == ST_F16S || storage == ST_BF16S;
+    t.shape = nr == 1 ? 0 : ((v < 2) != sixteen ? 1 : 0);
     t.zchunk = variant < nr ? 24 : 32;
     t.h = v % 2 ? 16 : 8;
     t.rows = tau1_strip_rows(storage, t.shape);

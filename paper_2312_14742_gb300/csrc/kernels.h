@@ -11,8 +11,8 @@ namespace lbm {
 
 // Tau1 step kernels (dense layout).
 cudaError_t launch_tau1_simple(int q, int storage, const StepArgs& a, cudaStream_t s);
-// Tiled kernel (tau1_strip.cu): variant v is strip shape v % R, R =
-// tau1_tile_shapes, with z chunks that fill whole waves, of 32, 16 or 48 planes (v / R).
+// Tiled kernel (tau1_strip.cu): variant v is shape choice v % R, R =
+// tau1_tile_shapes (0: by the box), with z chunks by the box, of 32, 16 or 48 planes (v / R).
 cudaError_t launch_tau1_tiled(int q, int storage, int variant, const StepArgs& a, cudaStream_t s);
 bool tau1_tiled_supported(int q, int storage, int64_t n);
 int tau1_tiled_variants(int q, int storage);
@@ -23,6 +23,7 @@ int tau1_tile_shapes(int storage);
 // chunk of zchunk planes. An owned column has its neighbours in the next lanes.
 // after_list: the last launch on s is launch_tau1_list() of the same step.
 constexpr int STRIP_ITEM = 33;
+constexpr int STRIP_WARPS = 4;  // warps per block of the dense and batched kernels, a strip each
 int tau1_strip_rows(int storage, int shape);
 cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
                                    int count, bool after_list, cudaStream_t s);

@@ -30,6 +30,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "pack2.cuh"
 #include "static_for.cuh"
 
 namespace lbm {
@@ -70,27 +71,64 @@ template <typename T> __device__ __forceinline__ Moments<T> moments_from(T d, T 
 // result can feed a packed sum, see above.
 template <typename T> __device__ __forceinline__ T product(T a, T b) { return fma(a, b, T(0)); }
 
-// V g in the compute precision.
-template <typename T> struct Force {
-    T x, y, z;
-    __device__ __forceinline__ explicit Force(const StepArgs& a)
-        : x(T(Scale<T>::V) * gcomp<T>(a, 0)), y(T(Scale<T>::V) * gcomp<T>(a, 1)), z(T(Scale<T>::V) * gcomp<T>(a, 2))
+// How a stored record enters its moments: V (u + g), R (1 + drho), drho. The
+// values of FP16 records come as stored, times their scales S_f; 1 / S_f is a
+// power of two and goes into the factors, which gives the same values.
+template <int ST> struct Terms {
+    using T = typename Storage<ST>::ctype;
+    static constexpr bool SCALED = ST == ST_F16S;
+    T gx, gy, gz;
+    T k[SCALED ? 5 : 1];
+    __device__ __forceinline__ Terms(const StepArgs& a, const Scales& sc)
+        : gx(T(Scale<T>::V) * gcomp<T>(a, 0)), gy(T(Scale<T>::V) * gcomp<T>(a, 1)), gz(T(Scale<T>::V) * gcomp<T>(a, 2))
     {
+        if constexpr (SCALED) {
+            k[0] = sc.inv[0];
+            k[1] = T(Scale<T>::R) * sc.inv[0];
+#pragma unroll
+            for (int f = 1; f < 4; ++f) k[f + 1] = T(Scale<T>::V) * sc.inv[f];
+        }
     }
+    template <int I> __device__ __forceinline__ T factor() const
+    {
+        if constexpr (SCALED) return k[I];
+        else return I == 0 ? T(1) : (I == 1 ? T(Scale<T>::R) : T(Scale<T>::V));
+    }
+    __device__ __forceinline__ T drho(T d) const { return SCALED ? factor<0>() * d : d; }
+    __device__ __forceinline__ T r(T d) const { return fma(factor<1>(), d, T(Scale<T>::R)); }
+    __device__ __forceinline__ T vx(T u) const { return fma(factor<2>(), u, gx); }
+    __device__ __forceinline__ T vy(T u) const { return fma(factor<3>(), u, gy); }
+    __device__ __forceinline__ T vz(T u) const { return fma(factor<4>(), u, gz); }
 };
 
-// Moments of one source record; a wall (solid) has none.
-template <typename T>
-__device__ __forceinline__ Moments<T> moments_of(T d, T ux, T uy, T uz, const Force<T>& g, bool solid)
+// Values of a record as stored, in the compute type.
+template <typename E> struct Rec {
+    E d, ux, uy, uz;
+};
+template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> record(const void* base, uint32_t i)
 {
-    const T d0 = solid ? T(0) : d;
-    const T r = solid ? T(0) : fma(T(Scale<T>::R), d, T(Scale<T>::R)), V = T(Scale<T>::V);
-    return moments_from<T>(d0, r, fma(V, ux, g.x), fma(V, uy, g.y), fma(V, uz, g.z));
+    const float one[4] = {1.f, 1.f, 1.f, 1.f};
+    Rec<typename Storage<ST>::ctype> r;
+    Storage<ST>::load(base, i, one, r.d, r.ux, r.uy, r.uz);
+    return r;
 }
-template <typename T>
-__device__ __forceinline__ Moments<T> moments_of_record(T d, T ux, T uy, T uz, const Force<T>& g)
+template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> record_at(const void* p)
 {
-    return moments_of<T>(d, ux, uy, uz, g, isnan(d));  // drho NaN: a solid node
+    const float one[4] = {1.f, 1.f, 1.f, 1.f};
+    Rec<typename Storage<ST>::ctype> r;
+    Storage<ST>::load_at(p, one, r.d, r.ux, r.uy, r.uz);
+    return r;
+}
+
+// Moments of one source record; a wall (solid) has none.
+template <int ST, typename T>
+__device__ __forceinline__ Moments<T> moments_of(const Rec<T>& c, const Terms<ST>& t, bool solid)
+{
+    return moments_from<T>(solid ? T(0) : t.drho(c.d), solid ? T(0) : t.r(c.d), t.vx(c.ux), t.vy(c.uy), t.vz(c.uz));
+}
+template <int ST, typename T> __device__ __forceinline__ Moments<T> moments_of_record(const Rec<T>& c, const Terms<ST>& t)
+{
+    return moments_of<ST, T>(c, t, isnan(c.d));  // drho NaN: a solid node
 }
 
 // c.v for a constant direction c (axis order x, y, z).
@@ -335,26 +373,19 @@ __device__ __forceinline__ void node_state(const T (&s)[4], T& d, T& ux, T& uy, 
     uz = s[3] * r;
 }
 
-// One record.
-template <typename E> struct Rec {
-    E d, ux, uy, uz;
-};
-
-// Moments of a pair of records in the lanes of L (f2 or d2, pack2.cuh); MIRROR
-// mirrors lane B in y. The solid bits come back in sA and sB.
-template <bool MIRROR, typename E, typename L>
-__device__ __forceinline__ Moments<L> pair_moments(const Rec<E>& a, const Rec<E>& b, const Force<E>& g, bool& sA,
-                                                   bool& sB)
+// Moments of a pair of records in the lanes of L (f2 or d2, pack2.cuh), solid
+// where sA or sB; MIRROR 1 (2) mirrors lane B in x (y), which gives the same
+// values with the directions exchanged.
+template <int MIRROR, int ST, typename L, typename E>
+__device__ __forceinline__ Moments<L> pair_moments(const Rec<E>& a, const Rec<E>& b, const Terms<ST>& t, bool sA, bool sB)
 {
-    sA = isnan(a.d);
-    sB = isnan(b.d);
-    const L d = L(sA ? E(0) : a.d, sB ? E(0) : b.d);
-    const E R = E(Scale<E>::R), V = E(Scale<E>::V);
-    const L r = L(sA ? E(0) : fma(R, a.d, R), sB ? E(0) : fma(R, b.d, R));
-    const L vx = L(fma(V, a.ux, g.x), fma(V, b.ux, g.x));
-    L vy = L(fma(V, a.uy, g.y), fma(V, b.uy, g.y));
-    const L vz = L(fma(V, a.uz, g.z), fma(V, b.uz, g.z));
-    if constexpr (MIRROR) vy.v.y = -vy.v.y;
+    const L d = L(sA ? E(0) : t.drho(a.d), sB ? E(0) : t.drho(b.d));
+    const L r = L(sA ? E(0) : t.r(a.d), sB ? E(0) : t.r(b.d));
+    L vx = L(t.vx(a.ux), t.vx(b.ux));
+    L vy = L(t.vy(a.uy), t.vy(b.uy));
+    const L vz = L(t.vz(a.uz), t.vz(b.uz));
+    if constexpr (MIRROR == 1) vx.v.y = -vx.v.y;
+    if constexpr (MIRROR == 2) vy.v.y = -vy.v.y;
     return moments_from<L>(d, r, vx, vy, vz);
 }
 
@@ -409,51 +440,85 @@ __device__ __forceinline__ void add_bounce(const Moments<T>& own, uint32_t wall,
     for (int f = 0; f < 4; ++f) s[f] = s[f] + B[f];
 }
 
-// The same update gathered by one thread: at(k) gives the moments of the source
-// x - c_k (k an integral constant, 0: the node itself).
+// The sums of one column of nine sources: at(dy, dz) gives their moments.
 template <int Q, typename T, typename F>
-__device__ __forceinline__ void gather_sums(F&& source, T (&s)[4])
+__device__ __forceinline__ void column_sums(F&& at, T (&X)[3], T (&Y)[3], T (&C)[3])
 {
     using S = Sums<Q>;
-    auto at = [&](auto xc, auto yc, auto zc) -> Moments<T> {
-        constexpr int K = kdir(-decltype(xc)::value, -decltype(yc)::value, -decltype(zc)::value);
-        if constexpr (K < Q) return source(std::integral_constant<int, K>{});
-        else return Moments<T>{};  // no such link: its values are not used
-    };
-    T X[3], Y[3], C[3];
-    static_for<0, 3>([&](auto xc) {
-        constexpr int DX = decltype(xc)::value - 1;
-        T P[S::NP], O[S::NO], M[S::NP];
-        static_for<0, 3>([&](auto zc) {
-            constexpr int DZ = decltype(zc)::value - 1;
-            using IX = std::integral_constant<int, DX>;
-            using IZ = std::integral_constant<int, DZ>;
-            typename S::template Mid<T> c, skip;
-            T up[S::NV], dn[S::NV], none[S::NV];
-            S::in_plane(at(IX{}, std::integral_constant<int, 0>{}, IZ{}), c, none, none);
-            S::in_plane(at(IX{}, std::integral_constant<int, -1>{}, IZ{}), skip, up, none);
-            S::in_plane(at(IX{}, std::integral_constant<int, 1>{}, IZ{}), skip, none, dn);
-            T p[S::NP], o[S::NO], m[S::NP];
-            S::y_sum(c, up, dn, p, o, m);
+    T P[S::NP], O[S::NO], M[S::NP];
+    static_for<0, 3>([&](auto zc) {
+        constexpr int DZ = decltype(zc)::value - 1;
+        using IZ = std::integral_constant<int, DZ>;
+        typename S::template Mid<T> c, skip;
+        T up[S::NV], dn[S::NV], none[S::NV];
+        S::in_plane(at(std::integral_constant<int, 0>{}, IZ{}), c, none, none);
+        S::in_plane(at(std::integral_constant<int, -1>{}, IZ{}), skip, up, none);
+        S::in_plane(at(std::integral_constant<int, 1>{}, IZ{}), skip, none, dn);
+        T p[S::NP], o[S::NO], m[S::NP];
+        S::y_sum(c, up, dn, p, o, m);
 #pragma unroll
-            for (int j = 0; j < S::NP; ++j) {
-                if (DZ == -1) P[j] = p[j];
-                if (DZ == 1) M[j] = m[j];
+        for (int j = 0; j < S::NP; ++j) {
+            if (DZ == -1) P[j] = p[j];
+            if (DZ == 1) M[j] = m[j];
+        }
+#pragma unroll
+        for (int j = 0; j < S::NO; ++j)
+            if (DZ == 0) O[j] = o[j];
+    });
+    T z[9];
+    S::z_begin(P, O, z);
+    S::z_end(z, M, X, Y, C);
+}
+
+// The same update gathered by one thread: fetch(k, solid) gives the record of the
+// source x - c_k and whether it is a wall, own the moments of the node itself. In
+// D3Q19 the columns on both sides share the lanes of packed arithmetic, the right
+// one mirrored in x (9.9 M listed nodes 221 us, 231 without); D3Q27 has no
+// registers for that (1.8 M sparse nodes 110 us, 74 without).
+template <int Q, int ST, typename T, typename F>
+__device__ __forceinline__ void gather_sums(const Terms<ST>& t, const Moments<T>& own, F&& fetch, T (&s)[4])
+{
+    T X[3], Y[3], C[3], skipA[3], skipB[3];
+    auto column = [&](auto xc, T (&X)[3], T (&Y)[3], T (&C)[3]) {
+        column_sums<Q, T>([&](auto yc, auto zc) -> Moments<T> {
+            constexpr int K = kdir(-decltype(xc)::value, -decltype(yc)::value, -decltype(zc)::value);
+            if constexpr (K == 0) {
+                return own;
+            } else if constexpr (K < Q) {
+                bool w;
+                const Rec<T> r = fetch(std::integral_constant<int, K>{}, w);
+                return moments_of<ST, T>(r, t, w);
+            } else {
+                return Moments<T>{};  // no such link: its values are not used
             }
-#pragma unroll
-            for (int j = 0; j < S::NO; ++j)
-                if (DZ == 0) O[j] = o[j];
-        });
-        T z[9], x[3], y[3], c[3];
-        S::z_begin(P, O, z);
-        S::z_end(z, M, x, y, c);
+        }, X, Y, C);
+    };
+    if constexpr (Q == 19) {
+        using L = typename Lanes<T>::type;
+        L sides[3], skipX[3], skipC[3];
+        column_sums<Q, L>([&](auto yc, auto zc) -> Moments<L> {
+            constexpr int K = kdir(1, -decltype(yc)::value, -decltype(zc)::value);
+            constexpr int KR = kdir(-1, -decltype(yc)::value, -decltype(zc)::value);
+            if constexpr (K < Q) {
+                bool sA, sB;
+                const Rec<T> a = fetch(std::integral_constant<int, K>{}, sA);
+                const Rec<T> b = fetch(std::integral_constant<int, KR>{}, sB);
+                return pair_moments<1, ST, L>(a, b, t, sA, sB);
+            } else {
+                return Moments<L>{};
+            }
+        }, sides, skipX, skipC);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            if (DX == -1) X[j] = x[j];
-            if (DX == 0) C[j] = c[j];
-            if (DX == 1) Y[j] = y[j];
+            X[j] = sides[j].v.x;
+            Y[j] = sides[j].v.y;
         }
-    });
+    } else {
+        column(std::integral_constant<int, -1>{}, X, skipA, skipB);
+    }
+    T skip[3];
+    column(std::integral_constant<int, 0>{}, skipA, skipB, C);
+    if constexpr (Q != 19) column(std::integral_constant<int, 1>{}, skipA, Y, skip);
     node_sums<Q, T>(C, X, Y, s);
 }
 

@@ -127,38 +127,35 @@ __global__ void __launch_bounds__(256) table_kernel(int nf, int nx, int ny, int 
 }
 
 // One Tau1 step of the fluid list: one thread per fluid node. D3Q19 hides the
-// latency of its gathers with warps (32 registers: 55.4 us for 1.8 M nodes, 61.2
+// latency of its gathers with warps (32 registers: 54.5 us for 1.8 M nodes, 61
 // with the registers the compiler would take); D3Q27 does better with more loads
-// in flight per thread (75.5 us against 94.8 at 40 registers).
+// in flight per thread (74 us against 95 at 40 registers). Summing link by link
+// took 55.5 and 82 us; in FP16 61.6 and 82, now 53.5 and 86.
 constexpr int sparse_blocks(int q, int st) { return q == 19 ? (st == ST_F64 ? 0 : 8) : (st == ST_F16S ? 4 : 0); }
 template <int Q, int ST>
 __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(StepArgs a, int nf, const int* __restrict__ nbr)
 {
-    using S = Storage<ST>;
-    using T = typename S::ctype;
+    using T = typename Storage<ST>::ctype;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf) return;
     const Scales sc(a.dscale);
-    const Force<T> g(a);
+    const Terms<ST> t(a, sc);
     // every index first: the records' loads then wait for none but their own
     int src[Q];
     static_for<1, Q>([&](auto kc) {
         constexpr int K = decltype(kc)::value;
         src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
     });
-    T d0, ux0, uy0, uz0;
-    S::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
-    const Moments<T> own = moments_of<T>(d0, ux0, uy0, uz0, g, false);
+    const Moments<T> own = moments_of<ST, T>(record<ST>(a.pre, (uint32_t)i), t, false);
     uint32_t wall = 0;
     T sums[4];
-    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
+    gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
         constexpr int K = decltype(kc)::value;
-        if constexpr (K == 0) return own;
-        const bool w = src[K] < 0;
-        T d = T(0), ux = T(0), uy = T(0), uz = T(0);
-        if (!w) S::load(a.pre, (uint32_t)src[K], sc.inv, d, ux, uy, uz);
-        if (w) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
-        return moments_of<T>(d, ux, uy, uz, g, w);
+        solid = src[K] < 0;
+        Rec<T> c{T(0), T(0), T(0), T(0)};
+        if (!solid) c = record<ST>(a.pre, (uint32_t)src[K]);
+        if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+        return c;
     }, sums);
     add_bounce<Q, T>(own, wall, sums);
 

@@ -24,7 +24,7 @@
 // non-periodic face keeps a NaN record.
 //
 // 256^3, spheres of radius 8 at 90% porosity: D3Q19 FP32 137 us per step (the
-// link-by-link row-pair kernel before it 155), BF16 158 (185), D3Q27 FP32 146
+// link-by-link row-pair kernel before it 155), BF16 153 (185), D3Q27 FP32 146
 // (247); 128^3 D3Q19 FP64 660 (937). FP32 is bound by issue and the latency
 // of its 12 warps per SM, not by HBM (74 us for the state alone). Blocks whose
 // four warps met at a barrier per plane and formed 32 own columns each took 149,
@@ -44,7 +44,7 @@ template <int Q, int ST, int R_> struct Cfg {
     using E = typename Storage<ST>::ctype;
     using L = typename Lanes<E>::type;
     using S = Sums<Q>;
-    static constexpr int W = 4, NT = 32 * W;                  // strips (warps) per block
+    static constexpr int W = STRIP_WARPS, NT = 32 * W;                  // strips (warps) per block
     static constexpr int R = R_, NP = R / 2;                  // rows and pairs of rows per strip
     static constexpr int REC = Storage<ST>::NODE_BYTES;
     static constexpr int NSTAGE = 3;                          // previous, current and next plane
@@ -181,7 +181,6 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
                                            unsigned char* smem, float (&amax)[4])
 {
     using C = Cfg<Q, ST, R_>;
-    using St = Storage<ST>;
     using E = typename C::E;
     using L = typename C::L;
     using S = Sums<Q>;
@@ -191,18 +190,21 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
     const int lane = threadIdx.x & 31;
     const uint32_t nxy = (uint32_t)a.nx * (uint32_t)a.ny;
     const size_t plane = (size_t)nxy * REC;
-    Force<E> g(a);
-    g.x = uniform(g.x);
-    g.y = uniform(g.y);
-    g.z = uniform(g.z);
+    Terms<ST> t(a, sc);
+    t.gx = uniform(t.gx);
+    t.gy = uniform(t.gy);
+    t.gz = uniform(t.gz);
+    float scale[4] = {1.f, 1.f, 1.f, 1.f};
+    if constexpr (t.SCALED) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) t.k[k] = uniform(t.k[k]);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) scale[f] = uniform(sc.s[f]);
+    }
 
     unsigned char* const mine = smem + lane * REC;
     auto cell = [&](int slot, int row) { return mine + slot * (B * C::LINE) + (row + 1) * C::LINE; };
-    auto read = [&](const unsigned char* p) {
-        Rec<E> r;
-        St::load_at(p, sc.inv, r.d, r.ux, r.uy, r.uz);
-        return r;
-    };
+    auto read = [&](const unsigned char* p) { return record_at<ST>(p); };
     // in-plane index of a staged cell's image in the box; false for a wall
     auto source = [&](int x, int y, uint32_t& xy) {
         const bool ok = wrap_coord(x, a.nx, a.periodic[0]) && wrap_coord(y, a.ny, a.periodic[1]);
@@ -270,9 +272,8 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
         if (lane >= half) return;
         const int eA = first + lane, eB = eA + half < end ? eA + half : eA;
         const uint4 iA = ids[eA], iB = ids[eB];
-        bool sA, sB;
         const Rec<E> rA = read(raw + eA * REC), rB = read(raw + eB * REC);
-        const Moments<L> m = pair_moments<false, E, L>(rA, rB, g, sA, sB);
+        const Moments<L> m = pair_moments<0, ST, L>(rA, rB, t, false, false);
         L s[4], Bn[4];
         bounce<Q, L>(m, [&](auto kc, L v, auto&& add) {
             // the source x - c_k: its column's word, its plane's bits, its row's bit
@@ -286,10 +287,10 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
         for (int f = 0; f < 4; ++f) s[f] = lanes_of(part[4 * eA + f], part[4 * eB + f]) + Bn[f];
         L d, ux, uy, uz;
         node_state<Q, L>(s, d, ux, uy, uz);
-        step_store<ST>(a.post, iA.x, d.v.x, ux.v.x, uy.v.x, uz.v.x, sc.s, a.seed);
+        step_store<ST>(a.post, iA.x, d.v.x, ux.v.x, uy.v.x, uz.v.x, scale, a.seed);
         if constexpr (AMAX) track_amax(amax, d.v.x, ux.v.x, uy.v.x, uz.v.x);
         if (eB != eA) {
-            step_store<ST>(a.post, iB.x, d.v.y, ux.v.y, uy.v.y, uz.v.y, sc.s, a.seed);
+            step_store<ST>(a.post, iB.x, d.v.y, ux.v.y, uy.v.y, uz.v.y, scale, a.seed);
             if constexpr (AMAX) track_amax(amax, d.v.y, ux.v.y, uy.v.y, uz.v.y);
         }
     };
@@ -317,16 +318,16 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
             {
                 L skip[NV];
                 typename S::template Mid<L> skipm;
-                bool sA, sB;
                 const Rec<E> ra = read(cell(slot, -1)), rb = read(cell(slot, R));
-                S::in_plane(pair_moments<true, E, L>(ra, rb, g, sA, sB), skipm, h, skip);
+                const bool sA = isnan(ra.d), sB = isnan(rb.d);
+                S::in_plane(pair_moments<2, ST, L>(ra, rb, t, sA, sB), skipm, h, skip);
                 sb |= (sA ? 1u : 0u) | (sB ? 2u << R : 0u);
             }
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
-                bool sA, sB;
                 const Rec<E> ra = read(cell(slot, j)), rb = read(cell(slot, j + NP));
-                S::in_plane(pair_moments<false, E, L>(ra, rb, g, sA, sB), mid[j], up[j], dn[j]);
+                const bool sA = isnan(ra.d), sB = isnan(rb.d);
+                S::in_plane(pair_moments<0, ST, L>(ra, rb, t, sA, sB), mid[j], up[j], dn[j]);
                 sb |= (sA ? 2u << j : 0u) | (sB ? 2u << (j + NP) : 0u);
             }
 #pragma unroll
@@ -393,11 +394,11 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
             L d, ux, uy, uz;
             node_state<Q, L>(s[j], d, ux, uy, uz);
             if (store >> (j + 1) & 1u) {
-                step_store<ST>(a.post, zoff + xy + (uint32_t)(j * a.nx), d.v.x, ux.v.x, uy.v.x, uz.v.x, sc.s, a.seed);
+                step_store<ST>(a.post, zoff + xy + (uint32_t)(j * a.nx), d.v.x, ux.v.x, uy.v.x, uz.v.x, scale, a.seed);
                 if constexpr (AMAX) track_amax(amax, d.v.x, ux.v.x, uy.v.x, uz.v.x);
             }
             if (store >> (j + NP + 1) & 1u) {
-                step_store<ST>(a.post, zoff + xy + (uint32_t)((j + NP) * a.nx), d.v.y, ux.v.y, uy.v.y, uz.v.y, sc.s, a.seed);
+                step_store<ST>(a.post, zoff + xy + (uint32_t)((j + NP) * a.nx), d.v.y, ux.v.y, uy.v.y, uz.v.y, scale, a.seed);
                 if constexpr (AMAX) track_amax(amax, d.v.y, ux.v.y, uy.v.y, uz.v.y);
             }
         }
@@ -407,16 +408,15 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
     finish_listed(0, waiting);
 }
 
-// Rows per warp, and resident blocks the register budget is sized for. The
-// dense and batched kernels take them in the order of dense_shape().
-template <int Q, typename E, int V> struct ColShape;
-template <int Q> struct ColShape<Q, float, 0> { static constexpr int R = 2, MINB = 4; };
-template <int Q> struct ColShape<Q, float, 1> { static constexpr int R = 4, MINB = 3; };
-template <int Q> struct ColShape<Q, float, 2> { static constexpr int R = 2, MINB = 3; };
-template <int Q> struct ColShape<Q, float, 3> { static constexpr int R = 4, MINB = 2; };
-template <int Q, int V> struct ColShape<Q, double, V> { static constexpr int R = 2, MINB = 2; };
-constexpr int COL_SHAPES = 4;  // FP32-arithmetic formats; FP64 has one
-constexpr int dense_shape(int v) { return v == 0 ? 1 : (v == 1 ? 0 : v); }
+// Rows per strip, and resident blocks the register budget is sized for. Four rows
+// form six rows' moments for four, two rows four for two, but two leave
+// registers for more warps.
+template <typename E, int V> struct StripShape;
+template <> struct StripShape<float, 0> { static constexpr int R = 2, MINB = 4; };
+template <> struct StripShape<float, 1> { static constexpr int R = 4, MINB = 3; };
+template <> struct StripShape<float, 2> { static constexpr int R = 4, MINB = 2; };
+template <int V> struct StripShape<double, V> { static constexpr int R = 2, MINB = 2; };
+constexpr int STRIP_SHAPES = 3;  // FP32-arithmetic formats; FP64 has one
 
 }  // namespace col
 

@@ -14,37 +14,35 @@ namespace lbm {
 template <int Q, int ST>
 __global__ void __launch_bounds__(256) tau1_simple_kernel(StepArgs a)
 {
-    using S = Storage<ST>;
-    using T = typename S::ctype;
+    using T = typename Storage<ST>::ctype;
     const int64_t n = (int64_t)a.nx * a.ny * a.nz;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
     const Scales sc(a.dscale);
-    T d0, ux0, uy0, uz0;
-    S::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
-    if (isnan(d0)) return;  // solid node
+    const Terms<ST> t(a, sc);
+    if (i >= n) return;
+    const Rec<T> c0 = record<ST>(a.pre, (uint32_t)i);
+    if (isnan(c0.d)) return;  // solid node
     const int x = (int)(i % a.nx);
     const int y = (int)((i / a.nx) % a.ny);
     const int z = (int)(i / ((int64_t)a.nx * a.ny));
-    const Force<T> g(a);
-    const Moments<T> own = moments_of_record<T>(d0, ux0, uy0, uz0, g);
+    const Moments<T> own = moments_of_record<ST>(c0, t);
     uint32_t wall = 0;
     T sums[4];
-    gather_sums<Q, T>([&](auto kc) -> Moments<T> {
+    gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
         constexpr int K = decltype(kc)::value;
-        if constexpr (K == 0) return own;
         int sx = x - cvel(K, 0), sy = y - cvel(K, 1), sz = z - cvel(K, 2);
         bool inside = true;
         if (sx < 0 || sx >= a.nx) { if (a.periodic[0]) sx = sx < 0 ? sx + a.nx : sx - a.nx; else inside = false; }
         if (sy < 0 || sy >= a.ny) { if (a.periodic[1]) sy = sy < 0 ? sy + a.ny : sy - a.ny; else inside = false; }
         if (sz < 0 || sz >= a.nz) { if (a.periodic[2]) sz = sz < 0 ? sz + a.nz : sz - a.nz; else inside = false; }
-        T d = T(NAN), ux = T(0), uy = T(0), uz = T(0);
+        Rec<T> c{T(NAN), T(0), T(0), T(0)};
         if (inside) {
             const int64_t s = (int64_t)sx + (int64_t)a.nx * ((int64_t)sy + (int64_t)a.ny * sz);
-            S::load(a.pre, (uint32_t)s, sc.inv, d, ux, uy, uz);
+            c = record<ST>(a.pre, (uint32_t)s);
         }
-        if (isnan(d)) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
-        return moments_of_record<T>(d, ux, uy, uz, g);
+        solid = isnan(c.d);
+        if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+        return c;
     }, sums);
     add_bounce<Q, T>(own, wall, sums);
 

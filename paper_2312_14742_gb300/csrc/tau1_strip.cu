@@ -2,6 +2,8 @@
 // chunk-major order so that those of a chunk run side by side and read each
 // other's outer rows from L2. Every size, periodicity and storage format takes
 // this kernel; the compact layout runs it over a list of strips.
+#include <cmath>
+
 #include "strip.cuh"
 
 namespace lbm {
@@ -13,11 +15,11 @@ using namespace col;
 // list (or NULL): per strip 32 slots, negative (~slot) where the lane does not own
 // its column, and the chunk; else the strips of the whole box, chunk-major.
 template <int Q, int ST, int R, int MINB>
-__global__ void __launch_bounds__(128, MINB)
+__global__ void __launch_bounds__(Cfg<Q, ST, R>::NT, 4 * MINB / Cfg<Q, ST, R>::W)
     tau1_strip_kernel(StepArgs a, int nstrips, int count, int chunk, const int* __restrict__ list)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = uniform((int)(threadIdx.x >> 5)), i = 4 * (int)blockIdx.x + warp;
+    const int warp = uniform((int)(threadIdx.x >> 5)), i = Cfg<Q, ST, R>::W * (int)blockIdx.x + warp;
     if (i >= count) return;
     Place pl;
     int c;
@@ -38,21 +40,59 @@ __global__ void __launch_bounds__(128, MINB)
     if (list) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Planes per block for a box of `tiles` tiles when the GPU holds `resident`
-// blocks: the chunk with the least (waves of blocks) x (planes a block forms),
-// a block forming two planes beside its own and about as much again to start.
-int whole_waves(int nz, long long tiles, long long resident)
+// Time of a step of nz planes in strips of a shape and chunk, up to a factor. A
+// chunk of c planes costs its strip c + 4 planes (two beside its own, and as
+// much again to start). plane[n] is the time of a plane on an SM with n resident
+// blocks: nearly n times one where the SM is full, latency below. In a wave or
+// two the fullest SM decides, and strips differ (walls); many waves even out,
+// but for the end of the last one.
+double step_cost(int nz, long long strips, int chunk, int sms, int minb, const double* plane)
 {
-    int best = nz;
-    long long best_cost = -1;
-    for (int n = 1; n <= nz;) {
-        const int chunk = (nz + n - 1) / n, used = (nz + chunk - 1) / chunk;
-        const long long cost = ((tiles * used + resident - 1) / resident) * (chunk + 4);
-        if (best_cost < 0 || cost < best_cost) {
-            best = chunk;
-            best_cost = cost;
+    const long long blocks = (strips * ((nz + chunk - 1) / chunk) + STRIP_WARPS - 1) / STRIP_WARPS;
+    const double waves = (double)blocks / (sms * minb);
+    if (waves <= 1) return (chunk + 4) * 1.15 * plane[(blocks + sms - 1) / sms];
+    return (chunk + 4) * plane[minb] * (waves <= 2.5 ? 1.15 * std::ceil(waves) : waves + 0.4);
+}
+
+// Time of a plane with 0 .. 4 resident blocks, by format and shape, fitted to
+// sweeps of shape and chunk over 11 boxes. Measured, in us, with four rows and
+// two: D3Q19 FP32 96^3 16.6 and 14.6, 250 x 130 x 90 34.7 and 33.0, 128^3 24.8 and
+// 26.3, 384^3 408 and 428; BF16 512 x 256 x 256 311 and 285; FP16 161 x 127 x 101
+// 32.6 and 28.8. Chunks: BF16 512 x 256 x 256 in two rows takes 285 in chunks of
+// 48 planes, 294 of 32, 312 of 16, 333 of 256 (one wave).
+constexpr double PLANE_F32[STRIP_SHAPES][5] = {{0, 0.95, 1.3, 1.7, 2.1}, {0, 1.6, 2.3, 3.0, 0}, {0, 1.6, 2.3, 0, 0}};
+constexpr double PLANE_16[STRIP_SHAPES][5] = {{0, 0.87, 1.2, 1.56, 1.93}, {0, 1.6, 2.3, 3.0, 0}, {0, 1.6, 2.3, 0, 0}};
+constexpr double PLANE_F64[5] = {0, 1.2, 2.0, 0, 0};
+
+struct Plan {
+    int shape, chunk;
+};
+
+// The shape (of first, first - 1 .. last) and chunk of the least cost.
+Plan plan_of(const StepArgs& a, int storage, int sms, int first, int last, int chunk)
+{
+    Plan best{first, chunk};
+    double least = -1;
+    for (int v = first; v >= last; --v) {
+        const int minb = storage == ST_F64 ? StripShape<double, 0>::MINB : (v == 0 ? 4 : (v == 1 ? 3 : 2));
+        const double* plane = storage == ST_F64 ? PLANE_F64 : (storage == ST_F32 ? PLANE_F32[v] : PLANE_16[v]);
+        const long long strips = strips_of(a.nx, a.ny, a.periodic[0], tau1_strip_rows(storage, v));
+        auto take = [&](int c) {
+            const double cost = step_cost(a.nz, strips, c, sms, minb, plane);
+            if (least < 0 || cost < least) {
+                best = {v, c};
+                least = cost;
+            }
+        };
+        if (chunk > 0) {
+            take(chunk);
+            continue;
         }
-        n = chunk == 1 ? nz + 1 : (nz + chunk - 2) / (chunk - 1);  // the next smaller chunk
+        for (int n = 1; n <= a.nz;) {
+            const int c = (a.nz + n - 1) / n;
+            take(c);
+            n = c == 1 ? a.nz + 1 : (a.nz + c - 2) / (c - 1);  // the next smaller chunk
+        }
     }
     return best;
 }
@@ -60,7 +100,7 @@ int whole_waves(int nz, long long tiles, long long resident)
 template <int Q, int ST, int V>
 cudaError_t launch_t(const StepArgs& a, int zchunk, cudaStream_t s, const int* list, int count, bool after_list)
 {
-    using Sh = ColShape<Q, typename Storage<ST>::ctype, V>;
+    using Sh = StripShape<typename Storage<ST>::ctype, V>;
     using C = Cfg<Q, ST, Sh::R>;
     static_assert(C::SMEM <= 227 * 1024, "shared memory of one block");
     auto kern = tau1_strip_kernel<Q, ST, Sh::R, Sh::MINB>;
@@ -68,15 +108,7 @@ cudaError_t launch_t(const StepArgs& a, int zchunk, cudaStream_t s, const int* l
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     const long long strips = strips_of(a.nx, a.ny, a.periodic[0], C::R);
-    int chunk = a.nz < zchunk ? a.nz : zchunk;
-    if (zchunk == 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, C::SMEM);
-        if (e != cudaSuccess) return e;
-        chunk = whole_waves(a.nz, strips, (long long)sms * C::W * (per_sm > 0 ? per_sm : 1));
-    }
+    const int chunk = a.nz < zchunk ? a.nz : zchunk;
     const int nchunks = (a.nz + chunk - 1) / chunk;
     const long long n = list ? (long long)count : strips * nchunks;
     if (n > 0x7fffffffLL - C::W) return cudaErrorInvalidConfiguration;
@@ -104,7 +136,6 @@ cudaError_t launch_s(int shape, int zchunk, const StepArgs& a, cudaStream_t s, c
         case 0: return launch_t<Q, ST, 0>(a, zchunk, s, list, count, after_list);
         case 1: return launch_t<Q, ST, 1>(a, zchunk, s, list, count, after_list);
         case 2: return launch_t<Q, ST, 2>(a, zchunk, s, list, count, after_list);
-        case 3: return launch_t<Q, ST, 3>(a, zchunk, s, list, count, after_list);
         default: return cudaErrorInvalidValue;
         }
     }
@@ -126,7 +157,7 @@ cudaError_t launch(int q, int storage, int shape, int zchunk, const StepArgs& a,
     }
 }
 
-constexpr int CHUNKS[4] = {0, 32, 16, 48};  // planes per block; 0: whole waves of blocks
+constexpr int CHUNKS[4] = {0, 32, 16, 48};  // planes per chunk; 0: by the box
 
 }  // namespace
 
@@ -135,21 +166,28 @@ bool tau1_tiled_supported(int q, int storage, int64_t n)
     return (q == 19 || q == 27) && storage >= ST_F64 && storage <= ST_BF16S && n > 0 && n < ((int64_t)1 << 31);
 }
 
-int tau1_tile_shapes(int storage) { return storage == ST_F64 ? 1 : COL_SHAPES; }
+int tau1_tile_shapes(int storage) { return storage == ST_F64 ? 1 : STRIP_SHAPES + 1; }
 
 int tau1_tiled_variants(int, int storage) { return 4 * tau1_tile_shapes(storage); }
 
 int tau1_strip_rows(int storage, int shape)
 {
-    if (storage == ST_F64) return ColShape<19, double, 0>::R;
-    return shape == 0 || shape == 2 ? ColShape<19, float, 0>::R : ColShape<19, float, 1>::R;
+    if (storage == ST_F64) return StripShape<double, 0>::R;
+    return shape == 0 ? StripShape<float, 0>::R : StripShape<float, 1>::R;
 }
 
 cudaError_t launch_tau1_tiled(int q, int storage, int variant, const StepArgs& a, cudaStream_t s)
 {
     const int nr = tau1_tile_shapes(storage);
     if (variant < 0 || variant >= 4 * nr) return cudaErrorInvalidValue;
-    return launch(q, storage, nr == 1 ? 0 : dense_shape(variant % nr), CHUNKS[variant / nr], a, s, nullptr, 0, false);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int v = variant % nr, chunk = CHUNKS[variant / nr];  // v 0: the shape by the box
+    const Plan p = v > 0 ? plan_of(a, storage, sms, v - 1, v - 1, chunk)
+                         : plan_of(a, storage, sms, storage == ST_F64 ? 0 : 1, 0, chunk);
+    return launch(q, storage, p.shape, p.chunk, a, s, nullptr, 0, false);
 }
 
 cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
