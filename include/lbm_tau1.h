@@ -71,7 +71,7 @@ typedef enum { LBM_F64 = 0, LBM_F32 = 1, LBM_F16S = 2, LBM_BF16S = 3 } lbm_stora
  * sparse layout is for the Tau1 scheme, boxes of fewer than 2^31 nodes; its
  * FP32 and FP64 results equal the dense kernels' bits. */
 /* COMPACT: the dense records, with each step's work split by tile column
- * (32 x H x 24 or 32 nodes, H = 8 or 16 by the variant chosen with
+ * (32 x H x 24 or 32 nodes, H = 8, 16 or 12 by the variant chosen with
  * lbm_tau1_set_variant, variant 0 by default): tile columns without
  * fluid are never read or written; those whose fluid fraction is at least the
  * threshold f* are stepped by the tiled kernel through a list; the fluid

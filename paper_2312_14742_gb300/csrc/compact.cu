@@ -270,7 +270,7 @@ CompactTiles compact_tiles(int storage, int variant)
     const bool sixteen = storage == ST_F16S || storage == ST_BF16S;
     t.shape = nr == 1 ? 0 : ((v < 2) != sixteen ? 1 : 0);
     t.zchunk = variant < nr ? 24 : 32;
-    t.h = v % 2 ? 16 : 8;
+    t.h = v == 1 ? 16 : (v == 3 ? 12 : 8);
     t.rows = tau1_strip_rows(storage, t.shape);
     return t;
 }

@@ -33,7 +33,7 @@ cudaError_t launch_selftest_timeout(unsigned int* timeouts, cudaStream_t s);
 
 // Compact porous layout (compact.cu): tile columns of 32 x h x zchunk nodes,
 // numbered chunk-major, then by rows of tiles (variant v of [0, 2R), R =
-// tau1_tile_shapes: h 8 or 16 for even or odd v, zchunk 24 below R, else 32;
+// tau1_tile_shapes: h 8, 16, 8, 12 by v % R, zchunk 24 below R, else 32;
 // stepped in strips of the given shape and rows); fluid counts per tile column,
 // and the fluid nodes of listed tile columns in row order at the given offsets.
 struct CompactTiles {
