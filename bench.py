@@ -173,7 +173,7 @@ def paper_baseline(args):
             "source": "Table tab:perf_comp, D2Q9 on 4000^2"}
 
 
-TILED_KERNEL_SOURCES = ("tau1_strip.cu", "strip.cuh", "moments.cuh", "mbarrier.cuh", "pack2.cuh", "common.cuh",
+TILED_KERNEL_SOURCES = ("tau1_strip.cu", "strip.cuh", "moments.cuh", "links.cuh", "tau1_node.cuh", "mbarrier.cuh", "pack2.cuh", "common.cuh",
                         "lattice.cuh", "static_for.cuh", "kernels.h")
 
 

@@ -308,7 +308,7 @@ lbm_status build_fluid_list(lbm_tau1* h)
 lbm_status build_compact(lbm_tau1* h)
 {
     const lbm_tau1_config& c = h->cfg;
-    h->ctile = compact_tiles(c.storage, h->variant);
+    h->ctile = compact_tiles(c.q, c.storage, h->variant);
     const CompactTiles& ct = h->ctile;
     const int64_t nb = compact_tile_columns(ct, c.nx, c.ny, c.nz);
     if (h->ccounted != h->variant) {

@@ -116,11 +116,16 @@ __global__ void __launch_bounds__(Cfg<Q, ST, R>::NT, 4 * MINB / Cfg<Q, ST, R>::W
         const int local = uniform(it - begin[lo]);
         const uint32_t c = (uint32_t)uniform((int)D.cur);
         const StepArgs a = uniform_args(D, c);
-        const Scales sc(AMAX ? D.scale[c] : nullptr, AMAX ? D.scale[c ^ 1] : nullptr);
         const int nstrips = uniform(D.nstrips), z0 = local / nstrips * chunk, z1 = min(a.nz, z0 + chunk);
         const Place pl = place_of_strip<R>(a, local % nstrips);
-        float amax[4] = {0.f, 0.f, 0.f, 0.f};
-        strip_step<Q, ST, R, AMAX>(a, sc, pl, z0, z1, smem + warp * Cfg<Q, ST, R>::WARP, amax);
+        unsigned char* const mine = smem + warp * Cfg<Q, ST, R>::WARP;
+        [[maybe_unused]] float amax[4] = {0.f, 0.f, 0.f, 0.f};
+        if constexpr (by_links(ST)) {
+            const Scales sc(AMAX ? D.scale[c] : nullptr, AMAX ? D.scale[c ^ 1] : nullptr);
+            strip_links<Q, ST, R, AMAX>(a, sc, pl, z0, z1, mine, amax);
+        } else {
+            strip_step<Q, ST, R>(a, pl, z0, z1, mine);
+        }
         if (AMAX && (D.step + 1) % BATCH_RESCALE_EVERY == 0) {
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
@@ -151,7 +156,7 @@ __global__ void __launch_bounds__(Cfg<Q, ST, R>::NT, 4 * MINB / Cfg<Q, ST, R>::W
 
 template <int Q, int ST, int V>
 struct BatchKernel {
-    using Sh = StripShape<typename Storage<ST>::ctype, V>;
+    using Sh = StripShape<Q, ST, V>;
     using C = Cfg<Q, ST, Sh::R>;
     static_assert(C::SMEM <= 227 * 1024, "shared memory of one block");
     static constexpr auto fn() { return tau1_batch_kernel<Q, ST, Sh::R, Sh::MINB>; }
@@ -176,8 +181,10 @@ struct BatchKernel {
     }
 };
 
-// Shape of variant 0; the others name one.
-constexpr int BATCH_SHAPE = 1;
+// Shape of variant 0; the others name one. The arguments that come from the table
+// take registers: the formats summed link by link take the shape that spills
+// nothing, or next to nothing.
+constexpr int batch_shape(int q, int st) { return st == ST_BF16S ? 0 : 1; }
 
 template <int Q, int ST>
 cudaError_t dispatch_v(int variant, bool prep, BatchTable* T, int& grid, int& rows, cudaStream_t s)
@@ -190,7 +197,7 @@ cudaError_t dispatch_v(int variant, bool prep, BatchTable* T, int& grid, int& ro
         return variant == 0 ? go(BatchKernel<Q, ST, 0>{}) : cudaErrorInvalidValue;
     } else {
         switch (variant) {
-        case 0: return go(BatchKernel<Q, ST, BATCH_SHAPE>{});
+        case 0: return go(BatchKernel<Q, ST, batch_shape(Q, ST)>{});
         case 1: return go(BatchKernel<Q, ST, 0>{});
         case 2: return go(BatchKernel<Q, ST, 1>{});
         case 3: return go(BatchKernel<Q, ST, 2>{});

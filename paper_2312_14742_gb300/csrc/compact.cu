@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "links.cuh"
 #include "moments.cuh"
 
 namespace lbm {
@@ -63,7 +64,7 @@ __device__ __forceinline__ void axis_sources(uint32_t c, uint32_t n, int st, boo
 // gathered from the dense state. A source outside a non-periodic face is read
 // from the sentinel record n (drho = NaN, u = 0) that follows the box in both
 // state copies, so that every source is a plain load and a wall is recognised by
-// its NaN alone. The sums are those of moments.cuh. One thread per node: two
+// its NaN alone. The sums are those of moments.cuh or links.cuh. One thread per node: two
 // nodes per thread in packed arithmetic take a third fewer instructions but
 // leave too few warps to hide the gathers (303 us against 256 on 9.9 M nodes).
 // Away from the faces, where all nodes of a warp are as a rule, the sources lie at
@@ -109,34 +110,47 @@ __global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12
     asm volatile("griddepcontrol.launch_dependents;");  // the tiled kernel of this step: other nodes
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const Scales sc(a.dscale);
-    const Terms<ST> terms(a, sc);
     const uint32_t sentinel = (uint32_t)a.nx * (uint32_t)a.ny * (uint32_t)a.nz;
-    auto bit = [](auto kc) {
-        constexpr int K = decltype(kc)::value;
-        return 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
-    };
     if (t >= l.count) return;
     Around A;
     const bool inner = A.set(a, l, (uint32_t)__ldg(l.nodes + t));
-    const Rec<T> own_record = record<ST>(a.pre, A.i);
-    if (isnan(own_record.d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
+    Rec<T> r[Q];
+    auto load = [&](Rec<T>& c, uint32_t i) { Storage<ST>::load(a.pre, i, sc.inv, c.d, c.ux, c.uy, c.uz); };
+    load(r[0], A.i);
+    if (isnan(r[0].d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
     auto step = [&](auto source) {
-        Rec<T> r[Q];
-        if constexpr (sizeof(T) == 4 && Q == 19)  // every load first (else as they are used, for registers)
-            static_for<1, Q>([&](auto kc) { r[decltype(kc)::value] = record<ST>(a.pre, source(kc)); });
-        const Moments<T> own = moments_of_record<ST>(own_record, terms);
-        uint32_t wall = 0;
-        T sums[4];
-        gather_sums<Q, ST>(terms, own, [&](auto kc, bool& solid) {
+        constexpr bool FIRST = sizeof(T) == 4 && (Q == 19 || by_links(ST));
+        if constexpr (FIRST)  // every load first (else as they are used, for registers)
+            static_for<1, Q>([&](auto kc) { load(r[decltype(kc)::value], source(kc)); });
+        auto fetch = [&](auto kc, bool& solid) -> const Rec<T>& {
             constexpr int K = decltype(kc)::value;
-            if constexpr (sizeof(T) == 8 || Q == 27) r[K] = record<ST>(a.pre, source(kc));
+            if constexpr (!FIRST) load(r[K], source(kc));
             solid = isnan(r[K].d);
-            if (solid) wall |= bit(kc);
             return r[K];
-        }, sums);
-        add_bounce<Q, T>(own, wall, sums);
+        };
         T d, ux, uy, uz;
-        node_state<Q, T>(sums, d, ux, uy, uz);
+        if constexpr (by_links(ST)) {
+            gather_links<Q, T>(a, r[0].d, r[0].ux, r[0].uy, r[0].uz, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
+                const Rec<T>& c = fetch(kc, solid);
+                d = c.d;
+                ux = c.ux;
+                uy = c.uy;
+                uz = c.uz;
+            }, d, ux, uy, uz);
+        } else {
+            const Terms<ST> terms(a);
+            const Moments<T> own = moments_of<ST, T>(r[0], terms, false);
+            uint32_t wall = 0;
+            T sums[4];
+            gather_sums<Q, ST>(terms, own, [&](auto kc, bool& solid) {
+                constexpr int K = decltype(kc)::value;
+                const Rec<T>& c = fetch(kc, solid);
+                if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+                return c;
+            }, sums);
+            add_bounce<Q, T>(own, wall, sums);
+            node_state<Q, T>(sums, d, ux, uy, uz);
+        }
         step_store<ST>(a.post, A.i, d, ux, uy, uz, sc.s, a.seed);
     };
     // away from the faces the sources are at fixed distances
@@ -261,17 +275,16 @@ TileGeo geo_of(const CompactTiles& t, int nx, int ny, int nz)
 
 }  // namespace
 
-CompactTiles compact_tiles(int storage, int variant)
+CompactTiles compact_tiles(int q, int storage, int variant)
 {
     const int nr = tau1_tile_shapes(storage);
     CompactTiles t;
     const int v = variant % nr;
-    // four rows per strip, but two in the 16-bit formats (by default) and for v 2, 3
-    const bool sixteen = storage == ST_F16S || storage == ST_BF16S;
-    t.shape = nr == 1 ? 0 : ((v < 2) != sixteen ? 1 : 0);
+    // four rows per strip, two for v 2, 3; link by link two, and another register budget for v 2, 3
+    t.shape = nr == 1 ? 0 : ((v < 2) != by_links(storage) ? 1 : 0);
     t.zchunk = variant < nr ? 24 : 32;
     t.h = v == 1 ? 16 : (v == 3 ? 12 : 8);
-    t.rows = tau1_strip_rows(storage, t.shape);
+    t.rows = tau1_strip_rows(q, storage, t.shape);
     return t;
 }
 

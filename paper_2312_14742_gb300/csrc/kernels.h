@@ -24,7 +24,7 @@ int tau1_tile_shapes(int storage);
 // after_list: the last launch on s is launch_tau1_list() of the same step.
 constexpr int STRIP_ITEM = 33;
 constexpr int STRIP_WARPS = 4;  // warps per block of the dense and batched kernels, a strip each
-int tau1_strip_rows(int storage, int shape);
+int tau1_strip_rows(int q, int storage, int shape);
 cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
                                    int count, bool after_list, cudaStream_t s);
 // Self-test (selftest.cu): one warp waits, bounded, on an mbarrier phase
@@ -39,7 +39,7 @@ cudaError_t launch_selftest_timeout(unsigned int* timeouts, cudaStream_t s);
 struct CompactTiles {
     int shape, zchunk, h, rows;
 };
-CompactTiles compact_tiles(int storage, int variant);
+CompactTiles compact_tiles(int q, int storage, int variant);
 int64_t compact_tile_columns(const CompactTiles& t, int nx, int ny, int nz);
 int64_t compact_tile_nodes(const CompactTiles& t, int nx, int ny, int nz, int b);
 // The strips that cover the given tile columns (in grid order), as

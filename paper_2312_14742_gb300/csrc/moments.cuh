@@ -1,4 +1,5 @@
-// Arithmetic of one Tau1 node update, shared by every 3D step kernel.
+// Arithmetic of one Tau1 node update in FP32 and FP64, shared by every 3D step
+// kernel (the 16-bit formats take links.cuh).
 //
 // Tau1 (Eq. LBMTau1) sums, over the directions k, the equilibrium of the
 // source x - c_k. With c_s^2 = 1/3 the equilibrium's deviation from its rest
@@ -22,7 +23,7 @@
 // its wall links. It is added to the finished sums, so a node without wall
 // links needs no wall arithmetic at all.
 //
-// Every kernel that steps a 3D node calls these functions in this order, with
+// Every kernel that steps such a node calls these functions in this order, with
 // every fused multiply-add written out, so all of them give the same bits. The
 // assembler fuses a packed product into a packed sum even where contraction is
 // off, so a product that feeds a sum is written product(): a fused operation
@@ -34,10 +35,6 @@
 #include "static_for.cuh"
 
 namespace lbm {
-
-// beside the two-lane overloads of pack2.cuh
-__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 template <typename T, typename = void> struct IsFp64 : std::is_same<T, double> {};
 template <typename T> struct IsFp64<T, std::void_t<typename T::elem>> : std::is_same<typename T::elem, double> {};
@@ -71,34 +68,18 @@ template <typename T> __device__ __forceinline__ Moments<T> moments_from(T d, T 
 // result can feed a packed sum, see above.
 template <typename T> __device__ __forceinline__ T product(T a, T b) { return fma(a, b, T(0)); }
 
-// How a stored record enters its moments: V (u + g), R (1 + drho), drho. The
-// values of FP16 records come as stored, times their scales S_f; 1 / S_f is a
-// power of two and goes into the factors, which gives the same values.
+// How a stored record enters its moments: V (u + g), R (1 + drho), drho.
 template <int ST> struct Terms {
     using T = typename Storage<ST>::ctype;
-    static constexpr bool SCALED = ST == ST_F16S;
     T gx, gy, gz;
-    T k[SCALED ? 5 : 1];
-    __device__ __forceinline__ Terms(const StepArgs& a, const Scales& sc)
+    __device__ __forceinline__ explicit Terms(const StepArgs& a)
         : gx(T(Scale<T>::V) * gcomp<T>(a, 0)), gy(T(Scale<T>::V) * gcomp<T>(a, 1)), gz(T(Scale<T>::V) * gcomp<T>(a, 2))
     {
-        if constexpr (SCALED) {
-            k[0] = sc.inv[0];
-            k[1] = T(Scale<T>::R) * sc.inv[0];
-#pragma unroll
-            for (int f = 1; f < 4; ++f) k[f + 1] = T(Scale<T>::V) * sc.inv[f];
-        }
     }
-    template <int I> __device__ __forceinline__ T factor() const
-    {
-        if constexpr (SCALED) return k[I];
-        else return I == 0 ? T(1) : (I == 1 ? T(Scale<T>::R) : T(Scale<T>::V));
-    }
-    __device__ __forceinline__ T drho(T d) const { return SCALED ? factor<0>() * d : d; }
-    __device__ __forceinline__ T r(T d) const { return fma(factor<1>(), d, T(Scale<T>::R)); }
-    __device__ __forceinline__ T vx(T u) const { return fma(factor<2>(), u, gx); }
-    __device__ __forceinline__ T vy(T u) const { return fma(factor<3>(), u, gy); }
-    __device__ __forceinline__ T vz(T u) const { return fma(factor<4>(), u, gz); }
+    __device__ __forceinline__ T r(T d) const { return fma(T(Scale<T>::R), d, T(Scale<T>::R)); }
+    __device__ __forceinline__ T vx(T u) const { return fma(T(Scale<T>::V), u, gx); }
+    __device__ __forceinline__ T vy(T u) const { return fma(T(Scale<T>::V), u, gy); }
+    __device__ __forceinline__ T vz(T u) const { return fma(T(Scale<T>::V), u, gz); }
 };
 
 // Values of a record as stored, in the compute type.
@@ -124,7 +105,7 @@ template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> re
 template <int ST, typename T>
 __device__ __forceinline__ Moments<T> moments_of(const Rec<T>& c, const Terms<ST>& t, bool solid)
 {
-    return moments_from<T>(solid ? T(0) : t.drho(c.d), solid ? T(0) : t.r(c.d), t.vx(c.ux), t.vy(c.uy), t.vz(c.uz));
+    return moments_from<T>(solid ? T(0) : c.d, solid ? T(0) : t.r(c.d), t.vx(c.ux), t.vy(c.uy), t.vz(c.uz));
 }
 template <int ST, typename T> __device__ __forceinline__ Moments<T> moments_of_record(const Rec<T>& c, const Terms<ST>& t)
 {
@@ -379,7 +360,7 @@ __device__ __forceinline__ void node_state(const T (&s)[4], T& d, T& ux, T& uy, 
 template <int MIRROR, int ST, typename L, typename E>
 __device__ __forceinline__ Moments<L> pair_moments(const Rec<E>& a, const Rec<E>& b, const Terms<ST>& t, bool sA, bool sB)
 {
-    const L d = L(sA ? E(0) : t.drho(a.d), sB ? E(0) : t.drho(b.d));
+    const L d = L(sA ? E(0) : a.d, sB ? E(0) : b.d);
     const L r = L(sA ? E(0) : t.r(a.d), sB ? E(0) : t.r(b.d));
     L vx = L(t.vx(a.ux), t.vx(b.ux));
     L vy = L(t.vy(a.uy), t.vy(b.uy));

@@ -70,6 +70,10 @@ __device__ __forceinline__ d2& operator+=(d2& a, d2 b) { a = a + b; return a; }
 __device__ __forceinline__ d2& operator-=(d2& a, d2 b) { a = a - b; return a; }
 __device__ __forceinline__ d2 recip(d2 x) { return d2(__drcp_rn(x.v.x), __drcp_rn(x.v.y)); }
 
+// scalars beside the two-lane overloads
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 template <typename E> struct Lanes;
 template <> struct Lanes<float> { using type = f2; };
 template <> struct Lanes<double> { using type = d2; };

@@ -12,9 +12,11 @@
 //   - the step reads the own record, the index and the source record of each
 //     link, and writes the own record: 2 (d+1) s + 4 (q-1) bytes per fluid
 //     node from HBM when the source records come from cache.
-// The arithmetic and its order are those of the dense kernels (moments.cuh), so
-// a sparse step gives the dense step's bits (FP32 and FP64).
+// The arithmetic and its order are those of the dense kernels (moments.cuh,
+// links.cuh), so a sparse step gives the dense step's bits (FP32 and FP64; 16-bit
+// stores round by the node's number, which is the list's here).
 #include "kernels.h"
+#include "links.cuh"
 #include "moments.cuh"
 
 namespace lbm {
@@ -130,8 +132,9 @@ __global__ void __launch_bounds__(256) table_kernel(int nf, int nx, int ny, int 
 // latency of its gathers with warps (32 registers: 54.5 us for 1.8 M nodes, 61
 // with the registers the compiler would take); D3Q27 does better with more loads
 // in flight per thread (74 us against 95 at 40 registers). Summing link by link
-// took 55.5 and 82 us; in FP16 61.6 and 82, now 53.5 and 86.
-constexpr int sparse_blocks(int q, int st) { return q == 19 ? (st == ST_F64 ? 0 : 8) : (st == ST_F16S ? 4 : 0); }
+// took 55.5 and 82 us, and does in FP16, where the order of the links stays
+// (links.cuh), 61.6 and 82.
+constexpr int sparse_blocks(int q, int st) { return q == 19 && st == ST_F32 ? 8 : 0; }
 template <int Q, int ST>
 __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(StepArgs a, int nf, const int* __restrict__ nbr)
 {
@@ -139,28 +142,38 @@ __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf) return;
     const Scales sc(a.dscale);
-    const Terms<ST> t(a, sc);
-    // every index first: the records' loads then wait for none but their own
-    int src[Q];
-    static_for<1, Q>([&](auto kc) {
-        constexpr int K = decltype(kc)::value;
-        src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
-    });
-    const Moments<T> own = moments_of<ST, T>(record<ST>(a.pre, (uint32_t)i), t, false);
-    uint32_t wall = 0;
-    T sums[4];
-    gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
-        constexpr int K = decltype(kc)::value;
-        solid = src[K] < 0;
-        Rec<T> c{T(0), T(0), T(0), T(0)};
-        if (!solid) c = record<ST>(a.pre, (uint32_t)src[K]);
-        if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
-        return c;
-    }, sums);
-    add_bounce<Q, T>(own, wall, sums);
-
     T d, ux, uy, uz;
-    node_state<Q, T>(sums, d, ux, uy, uz);
+    if constexpr (by_links(ST)) {
+        T d0, ux0, uy0, uz0;
+        Storage<ST>::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
+        gather_links<Q, T>(a, d0, ux0, uy0, uz0, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
+            constexpr int K = decltype(kc)::value;
+            const int j = __ldg(nbr + (int64_t)(K - 1) * nf + i);
+            solid = j < 0;
+            d = ux = uy = uz = T(0);
+            if (!solid) Storage<ST>::load(a.pre, (uint32_t)j, sc.inv, d, ux, uy, uz);
+        }, d, ux, uy, uz);
+    } else {
+        const Terms<ST> t(a);
+        int src[Q];
+        static_for<1, Q>([&](auto kc) {
+            constexpr int K = decltype(kc)::value;
+            src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
+        });
+        const Moments<T> own = moments_of<ST, T>(record<ST>(a.pre, (uint32_t)i), t, false);
+        uint32_t wall = 0;
+        T sums[4];
+        gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
+            constexpr int K = decltype(kc)::value;
+            solid = src[K] < 0;
+            Rec<T> c{T(0), T(0), T(0), T(0)};
+            if (!solid) c = record<ST>(a.pre, (uint32_t)src[K]);
+            if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+            return c;
+        }, sums);
+        add_bounce<Q, T>(own, wall, sums);
+        node_state<Q, T>(sums, d, ux, uy, uz);
+    }
     step_store<ST>(a.post, (uint32_t)i, d, ux, uy, uz, sc.s, a.seed);
 }
 

@@ -23,15 +23,19 @@
 // ragged boxes are just other addresses, and a cell that lies beyond a
 // non-periodic face keeps a NaN record.
 //
+// The 16-bit formats march the same strips link by link (strip_links()): no list,
+// and more values along x.
+//
 // 256^3, spheres of radius 8 at 90% porosity: D3Q19 FP32 137 us per step (the
-// link-by-link row-pair kernel before it 155), BF16 153 (185), D3Q27 FP32 146
-// (247); 128^3 D3Q19 FP64 660 (937). FP32 is bound by issue and the latency
+// link-by-link row-pair kernel before it 155), BF16 150 (183), D3Q27 FP32 146
+// (247), BF16 206 (315); 128^3 D3Q19 FP64 660 (937). FP32 is bound by issue and the latency
 // of its 12 warps per SM, not by HBM (74 us for the state alone). Blocks whose
 // four warps met at a barrier per plane and formed 32 own columns each took 149,
 // 173, 175 and 729.
 #pragma once
 
 #include "kernels.h"
+#include "links.cuh"
 #include "mbarrier.cuh"
 #include "moments.cuh"
 #include "pack2.cuh"
@@ -56,7 +60,7 @@ template <int Q, int ST, int R_> struct Cfg {
     static constexpr int PART = NSTAGE * B * LINE;            // [CAP][4]
     static constexpr int RAW = PART + CAP * 4 * (int)sizeof(E);
     static constexpr int IDS = RAW + (CAP * REC + 15) / 16 * 16;  // [CAP] x 16 bytes
-    static constexpr int WARP = IDS + CAP * 16;
+    static constexpr int WARP = by_links(ST) ? PART : IDS + CAP * 16;
     static constexpr int SMEM = W * WARP;
     static_assert(R % 2 == 0 && 3 * B <= 32, "rows");
     static_assert(PART % 16 == 0 && RAW % 16 == 0 && WARP % 16 == 0, "alignment");
@@ -121,12 +125,12 @@ __device__ __forceinline__ bool wrap_coord(int& c, int n, int periodic)
     return true;
 }
 
-template <typename E> __device__ __forceinline__ void track_amax(float (&m)[4], E d, E ux, E uy, E uz)
+__device__ __forceinline__ void track_amax(float (&m)[4], float d, float ux, float uy, float uz)
 {
-    m[0] = fmaxf(m[0], fabsf((float)d));
-    m[1] = fmaxf(m[1], fabsf((float)ux));
-    m[2] = fmaxf(m[2], fabsf((float)uy));
-    m[3] = fmaxf(m[3], fabsf((float)uz));
+    m[0] = fmaxf(m[0], fabsf(d));
+    m[1] = fmaxf(m[1], fabsf(ux));
+    m[2] = fmaxf(m[2], fabsf(uy));
+    m[3] = fmaxf(m[3], fabsf(uz));
 }
 
 // What a lane of a strip holds: the column at x and rows y0 .. y0 + R - 1; owner:
@@ -172,71 +176,61 @@ __host__ __device__ __forceinline__ long long strips_of(int nx, int ny, int peri
     return rotates(nx, periodic) ? rows : (rows * ((long long)nx + 2) - 2 + 29) / 30;
 }
 
-// One strip of one step: planes z0 <= z < z1 of the columns at pl. All lanes of
-// the warp call it together; smem holds Cfg::WARP bytes of this warp's own,
-// 16-byte aligned. With AMAX, amax[f] collects the largest |value| of field f
-// among the nodes this lane stores.
-template <int Q, int ST, int R_, bool AMAX>
-__device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, const Place& pl, int z0, int z1,
-                                           unsigned char* smem, float (&amax)[4])
-{
-    using C = Cfg<Q, ST, R_>;
-    using E = typename C::E;
-    using L = typename C::L;
-    using S = Sums<Q>;
-    constexpr int REC = C::REC, R = C::R, NP = C::NP, NV = S::NV;
-    constexpr int B = C::B;
-
-    const int lane = threadIdx.x & 31;
-    const uint32_t nxy = (uint32_t)a.nx * (uint32_t)a.ny;
-    const size_t plane = (size_t)nxy * REC;
-    Terms<ST> t(a, sc);
-    t.gx = uniform(t.gx);
-    t.gy = uniform(t.gy);
-    t.gz = uniform(t.gz);
-    float scale[4] = {1.f, 1.f, 1.f, 1.f};
-    if constexpr (t.SCALED) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) t.k[k] = uniform(t.k[k]);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) scale[f] = uniform(sc.s[f]);
-    }
-
-    unsigned char* const mine = smem + lane * REC;
-    auto cell = [&](int slot, int row) { return mine + slot * (B * C::LINE) + (row + 1) * C::LINE; };
-    auto read = [&](const unsigned char* p) { return record_at<ST>(p); };
-    // in-plane index of a staged cell's image in the box; false for a wall
-    auto source = [&](int x, int y, uint32_t& xy) {
-        const bool ok = wrap_coord(x, a.nx, a.periodic[0]) && wrap_coord(y, a.ny, a.periodic[1]);
-        xy = (uint32_t)x + (uint32_t)a.nx * (uint32_t)y;
-        return ok;
-    };
+// The planes of a strip as they pass through a warp's shared memory: R + 2 rows
+// of 32 records, a slot per plane, each lane's cells copied by the lane itself.
+// A cell beyond a non-periodic face holds a wall's record.
+template <int Q, int ST, int R> struct Planes {
+    using C = Cfg<Q, ST, R>;
+    static constexpr int REC = C::REC, B = C::B;
+    const StepArgs& a;
+    unsigned char* mine;
+    uint32_t nxy;
+    size_t plane;
     // the lane's cells: rows 0 .. rows - 1 are the box's, one plane row after
     // the other; row `rows` (above the strip, or the first one beyond the box in
     // its last strip) and row -1 are images of others, or walls
-    const int rows = min(R, a.ny - pl.y0);
+    int rows;
     uint32_t xy, xy_below, xy_above;
-    uint32_t ok = 0;  // bit r + 1: row r is copied
-    if (rows > 0) {
-        if (source(pl.x, pl.y0 - 1, xy_below)) ok |= 1u;
-        if (source(pl.x, pl.y0, xy))
-#pragma unroll
-            for (int r = 0; r < R; ++r) ok |= r < rows ? 2u << r : 0u;
-        if (source(pl.x, pl.y0 + rows, xy_above)) ok |= 2u << rows;
-    }
-    const bool full = __all_sync(0xffffffffu, ok == (1u << B) - 1u);
+    uint32_t ok = 0;      // bit r + 1: row r is copied
     uint32_t active = 0;  // bit r + 1: row r is a node this lane owns
-#pragma unroll
-    for (int r = 0; r < R; ++r) active |= pl.owner && r < rows ? 2u << r : 0u;
+    bool full;
 
-    __syncwarp();  // the previous call's last reads are done
-#pragma unroll
-    for (int s = 0; s < C::NSTAGE; ++s) {
-#pragma unroll
-        for (int r = 0; r < B; ++r)
-            if (!(ok >> r & 1u)) put_wall<ST>(cell(s, r - 1));
+    // in-plane index of a staged cell's image in the box; false for a wall
+    __device__ __forceinline__ bool source(int x, int y, uint32_t& i) const
+    {
+        const bool in = wrap_coord(x, a.nx, a.periodic[0]) && wrap_coord(y, a.ny, a.periodic[1]);
+        i = (uint32_t)x + (uint32_t)a.nx * (uint32_t)y;
+        return in;
     }
-    auto stage = [&](int p, int slot) {
+    __device__ __forceinline__ unsigned char* cell(int slot, int row) const
+    {
+        return mine + slot * (B * C::LINE) + (row + 1) * C::LINE;
+    }
+    __device__ __forceinline__ Planes(const StepArgs& args, const Place& pl, unsigned char* smem)
+        : a(args), mine(smem + (threadIdx.x & 31) * REC), nxy((uint32_t)args.nx * (uint32_t)args.ny),
+          plane((size_t)nxy * REC), rows(min(R, args.ny - pl.y0))
+    {
+        if (rows > 0) {
+            if (source(pl.x, pl.y0 - 1, xy_below)) ok |= 1u;
+            if (source(pl.x, pl.y0, xy))
+#pragma unroll
+                for (int r = 0; r < R; ++r) ok |= r < rows ? 2u << r : 0u;
+            if (source(pl.x, pl.y0 + rows, xy_above)) ok |= 2u << rows;
+        }
+        full = __all_sync(0xffffffffu, ok == (1u << B) - 1u);
+#pragma unroll
+        for (int r = 0; r < R; ++r) active |= pl.owner && r < rows ? 2u << r : 0u;
+        __syncwarp();  // the previous call's last reads are done
+#pragma unroll
+        for (int s = 0; s < C::NSTAGE; ++s) {
+#pragma unroll
+            for (int r = 0; r < B; ++r)
+                if (!(ok >> r & 1u)) put_wall<ST>(cell(s, r - 1));
+        }
+    }
+    // starts the copy of plane p into a slot
+    __device__ __forceinline__ void stage(int p, int slot) const
+    {
         int gz = p;
         if (wrap_coord(gz, a.nz, a.periodic[2])) {
             const unsigned char* base = static_cast<const unsigned char*>(a.pre) + (size_t)gz * plane;
@@ -259,7 +253,32 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
             for (int r = 0; r < B; ++r) put_wall<ST>(cell(slot, r - 1));
         }
         cp_commit();
-    };
+    }
+};
+
+// One strip of one step: planes z0 <= z < z1 of the columns at pl. All lanes of
+// the warp call it together; smem holds Cfg::WARP bytes of this warp's own,
+// 16-byte aligned.
+template <int Q, int ST, int R_>
+__device__ __forceinline__ void strip_step(const StepArgs& a, const Place& pl, int z0, int z1, unsigned char* smem)
+{
+    using C = Cfg<Q, ST, R_>;
+    using E = typename C::E;
+    using L = typename C::L;
+    using S = Sums<Q>;
+    constexpr int REC = C::REC, R = C::R, NP = C::NP, NV = S::NV;
+    constexpr int B = C::B;
+
+    const int lane = threadIdx.x & 31;
+    const uint32_t nxy = (uint32_t)a.nx * (uint32_t)a.ny;
+    Terms<ST> t(a);
+    t.gx = uniform(t.gx);
+    t.gy = uniform(t.gy);
+    t.gz = uniform(t.gz);
+
+    const Planes<Q, ST, R_> planes(a, pl, smem);
+    auto read = [&](const unsigned char* p) { return record_at<ST>(p); };
+    const uint32_t xy = planes.xy, active = planes.active;
 
     E* const part = reinterpret_cast<E*>(smem + C::PART);
     unsigned char* const raw = smem + C::RAW;
@@ -287,11 +306,9 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
         for (int f = 0; f < 4; ++f) s[f] = lanes_of(part[4 * eA + f], part[4 * eB + f]) + Bn[f];
         L d, ux, uy, uz;
         node_state<Q, L>(s, d, ux, uy, uz);
-        step_store<ST>(a.post, iA.x, d.v.x, ux.v.x, uy.v.x, uz.v.x, scale, a.seed);
-        if constexpr (AMAX) track_amax(amax, d.v.x, ux.v.x, uy.v.x, uz.v.x);
+        step_store<ST>(a.post, iA.x, d.v.x, ux.v.x, uy.v.x, uz.v.x, nullptr, a.seed);
         if (eB != eA) {
-            step_store<ST>(a.post, iB.x, d.v.y, ux.v.y, uy.v.y, uz.v.y, scale, a.seed);
-            if constexpr (AMAX) track_amax(amax, d.v.y, ux.v.y, uy.v.y, uz.v.y);
+            step_store<ST>(a.post, iB.x, d.v.y, ux.v.y, uy.v.y, uz.v.y, nullptr, a.seed);
         }
     };
 
@@ -302,11 +319,11 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
     uint32_t hist = 0;
     constexpr uint32_t HMASK = (1u << (3 * B)) - 1u;
     int slot = 0;
-    stage(z0 - 1, 0);
+    planes.stage(z0 - 1, 0);
 #pragma unroll 2
     for (int p = z0 - 1; p <= z1; ++p) {
         const int next = slot == C::NSTAGE - 1 ? 0 : slot + 1;
-        if (p < z1) stage(p + 1, next);
+        if (p < z1) planes.stage(p + 1, next);
         else cp_commit();
         cp_wait<1>();
         // y sums of the strip's pairs of rows, and the z sums of plane p - 1
@@ -318,14 +335,14 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
             {
                 L skip[NV];
                 typename S::template Mid<L> skipm;
-                const Rec<E> ra = read(cell(slot, -1)), rb = read(cell(slot, R));
+                const Rec<E> ra = read(planes.cell(slot, -1)), rb = read(planes.cell(slot, R));
                 const bool sA = isnan(ra.d), sB = isnan(rb.d);
                 S::in_plane(pair_moments<2, ST, L>(ra, rb, t, sA, sB), skipm, h, skip);
                 sb |= (sA ? 1u : 0u) | (sB ? 2u << R : 0u);
             }
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
-                const Rec<E> ra = read(cell(slot, j)), rb = read(cell(slot, j + NP));
+                const Rec<E> ra = read(planes.cell(slot, j)), rb = read(planes.cell(slot, j + NP));
                 const bool sA = isnan(ra.d), sB = isnan(rb.d);
                 S::in_plane(pair_moments<0, ST, L>(ra, rb, t, sA, sB), mid[j], up[j], dn[j]);
                 sb |= (sA ? 2u << j : 0u) | (sB ? 2u << (j + NP) : 0u);
@@ -372,7 +389,7 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
                     E* q = part + 4 * e;
 #pragma unroll
                     for (int f = 0; f < 4; ++f) q[f] = r < NP ? s[r % NP][f].v.x : s[r % NP][f].v.y;
-                    const unsigned char* rec = cell(slot == 0 ? C::NSTAGE - 1 : slot - 1, r);
+                    const unsigned char* rec = planes.cell(slot == 0 ? C::NSTAGE - 1 : slot - 1, r);
 #pragma unroll
                     for (int k = 0; k < REC / 8; ++k)
                         reinterpret_cast<uint2*>(raw + e * REC)[k] = reinterpret_cast<const uint2*>(rec)[k];
@@ -394,12 +411,10 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
             L d, ux, uy, uz;
             node_state<Q, L>(s[j], d, ux, uy, uz);
             if (store >> (j + 1) & 1u) {
-                step_store<ST>(a.post, zoff + xy + (uint32_t)(j * a.nx), d.v.x, ux.v.x, uy.v.x, uz.v.x, scale, a.seed);
-                if constexpr (AMAX) track_amax(amax, d.v.x, ux.v.x, uy.v.x, uz.v.x);
+                step_store<ST>(a.post, zoff + xy + (uint32_t)(j * a.nx), d.v.x, ux.v.x, uy.v.x, uz.v.x, nullptr, a.seed);
             }
             if (store >> (j + NP + 1) & 1u) {
-                step_store<ST>(a.post, zoff + xy + (uint32_t)((j + NP) * a.nx), d.v.y, ux.v.y, uy.v.y, uz.v.y, scale, a.seed);
-                if constexpr (AMAX) track_amax(amax, d.v.y, ux.v.y, uy.v.y, uz.v.y);
+                step_store<ST>(a.post, zoff + xy + (uint32_t)((j + NP) * a.nx), d.v.y, ux.v.y, uy.v.y, uz.v.y, nullptr, a.seed);
             }
         }
         slot = next;
@@ -408,14 +423,184 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Scales& sc, 
     finish_listed(0, waiting);
 }
 
+// The same strip in the 16-bit formats, summed link by link (links.cuh). What a
+// plane sends along x is shuffled per link. The sums of a node begin with the
+// c_z = +1 links, whose values wait in registers for the node's own plane, and
+// end with the c_z = -1 links, for which the node's own c_z = +1 values wait; wall
+// links take the node's own value in their place in the order, where the warp sees
+// any. With AMAX, amax[f] collects the largest |value| of field f among the
+// nodes this lane stores.
+template <int Q, int ST, int R_, bool AMAX>
+__device__ __forceinline__ void strip_links(const StepArgs& a, const Scales& sc, const Place& pl, int z0, int z1,
+                                            unsigned char* smem, float (&amax)[4])
+{
+    using C = Cfg<Q, ST, R_>;
+    using E = typename C::E;
+    using L = typename C::L;
+    constexpr int R = C::R, NP = C::NP, B = C::B, NC = Weights<Q>::NCLASS;
+
+    const uint32_t nxy = (uint32_t)a.nx * (uint32_t)a.ny;
+    const L g0(uniform(gcomp<E>(a, 0))), g1(uniform(gcomp<E>(a, 1))), g2(uniform(gcomp<E>(a, 2)));
+    float scale[4], inv[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        scale[f] = uniform(sc.s[f]);
+        inv[f] = uniform(sc.inv[f]);
+    }
+    const Planes<Q, ST, R_> planes(a, pl, smem);
+    const uint32_t xy = planes.xy, active = planes.active;
+
+    // outgoing values of two records, those of direction k and inv(k) from one
+    // product; none from a wall; MIRROR: the second record mirrored in y
+    auto outgoing = [&](const unsigned char* pa, const unsigned char* pb, auto mirror, L (&out)[Q], bool& sA, bool& sB) {
+        constexpr bool MIRROR = decltype(mirror)::value;
+        Rec<E> ra, rb;
+        Storage<ST>::load_at(pa, inv, ra.d, ra.ux, ra.uy, ra.uz);
+        Storage<ST>::load_at(pb, inv, rb.d, rb.ux, rb.uy, rb.uz);
+        sA = isnan(ra.d);
+        sB = isnan(rb.d);
+        const L d(sA ? E(0) : ra.d, sB ? E(0) : rb.d);
+        const L rho = L(E(1)) + d, mass(sA ? E(0) : rho.v.x, sB ? E(0) : rho.v.y);
+        const L vx = L(ra.ux, rb.ux) + g0, vz = L(ra.uz, rb.uz) + g2;
+        L vy = L(ra.uy, rb.uy) + g1;
+        if constexpr (MIRROR) vy.v.y = -vy.v.y;
+        const L vv = fma(vz, vz, fma(vy, vy, vx * vx));
+        const L A = fma(L(E(-1.5)) * mass, vv, d), r3 = L(E(3)) * mass, H = L(E(0.5)) * recip(rho);
+        const L Px = product(r3, vx), Py = product(r3, vy), Pz = product(r3, vz);
+        out[0] = A;
+        static_for<0, (Q - 1) / 2>([&](auto ic) {
+            constexpr int K = 1 + 2 * decltype(ic)::value;  // K + 1 = inv(K)
+            const L p = dir_dot<K, L>(Px, Py, Pz), e = fma(p * H, p, A);
+            out[K] = e + p;
+            out[K + 1] = e - p;
+        });
+    };
+
+    NodeAcc<L, NC> acc[NP];  // of plane p - 1, all but its c_z = -1 links
+    L up[NP][Q];             // c_z = +1 links: what they bring to plane p
+    L own[NP][Q];            // own c_z = +1 values of plane p - 1
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        acc[j].clear();
+#pragma unroll
+        for (int k = 0; k < Q; ++k) up[j][k] = own[j][k] = L(E(0));
+    }
+    // solid bits of this column and of those left and right: rows -1 .. R of planes p, p - 1, p - 2 (B bits each)
+    uint32_t hist = 0, hl = 0, hr = 0;
+    constexpr uint32_t HMASK = (1u << (3 * B)) - 1u;
+    int slot = 0;
+    planes.stage(z0 - 1, 0);
+#pragma unroll 1
+    for (int p = z0 - 1; p <= z1; ++p) {
+        const int next = slot == C::NSTAGE - 1 ? 0 : slot + 1;
+        if (p < z1) planes.stage(p + 1, next);
+        else cp_commit();
+        cp_wait<1>();
+        L out[NP][Q], edge[Q];  // edge: rows -1 and R, the latter mirrored in y
+        uint32_t sb = 0;
+        {
+            bool sA, sB;
+            outgoing(planes.cell(slot, -1), planes.cell(slot, R), std::true_type{}, edge, sA, sB);
+            sb |= (sA ? 1u : 0u) | (sB ? 2u << R : 0u);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                outgoing(planes.cell(slot, j), planes.cell(slot, j + NP), std::false_type{}, out[j], sA, sB);
+                sb |= (sA ? 2u << j : 0u) | (sB ? 2u << (j + NP) : 0u);
+            }
+        }
+        hist = (hist << B | sb) & HMASK;
+        const bool walls = __any_sync(0xffffffffu, hist != 0u);
+        if (walls) {
+            hl = __shfl_sync(0xffffffffu, hist, pl.left);
+            hr = __shfl_sync(0xffffffffu, hist, pl.right);
+        }
+        // what link k brings from plane p to the rows of pair j
+        auto brings = [&](auto kc, int j) -> L {
+            constexpr int K = decltype(kc)::value, cx = cvel(K, 0), cy = cvel(K, 1);
+            constexpr int KM = kdir(cx, -cy, cvel(K, 2));
+            L v = out[j][K];
+            if constexpr (cy == 1) v = j > 0 ? out[j > 0 ? j - 1 : 0][K] : lanes_of(edge[K].v.x, out[NP - 1][K].v.x);
+            if constexpr (cy == -1) v = j < NP - 1 ? out[j < NP - 1 ? j + 1 : 0][K] : lanes_of(out[0][K].v.y, edge[KM].v.y);
+            if constexpr (cx != 0) v = shfl_pair(v, cx == 1 ? pl.left : pl.right);
+            return v;
+        };
+        // v, or b where link k comes from a wall; PLANE: planes between its source and plane p
+        auto or_wall = [&](auto kc, auto plane, int j, L v, L b) -> L {
+            constexpr int K = decltype(kc)::value, cx = cvel(K, 0), PLANE = decltype(plane)::value;
+            const uint32_t w = cx == 1 ? hl : (cx == 0 ? hist : hr);
+            const uint32_t bit = 1u << (PLANE * B + 1 - cvel(K, 1));
+            return lanes_of(w & bit << j ? b.v.x : v.v.x, w & bit << (j + NP) ? b.v.y : v.v.y);
+        };
+        using Here = std::integral_constant<int, 0>;
+        using Below = std::integral_constant<int, 1>;
+        // plane p - 1: its last links; rows to store: fluid nodes of the box and the chunk
+        const uint32_t store = p > z0 ? active & ~(hist >> B) : 0u;
+        const uint32_t zoff = nxy * (uint32_t)(p - 1);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            L v[Q];
+            links_of<Q, -1>([&](auto kc) { v[decltype(kc)::value] = brings(kc, j); });
+            if (walls)
+                links_of<Q, -1>([&](auto kc) {
+                    constexpr int K = decltype(kc)::value;
+                    v[K] = or_wall(kc, Here{}, j, v[K], own[j][inv_dir(K)]);
+                });
+            links_of<Q, -1>([&](auto kc) { acc[j].template add<Q, decltype(kc)::value>(v[decltype(kc)::value]); });
+            L d, ux, uy, uz;
+            node_finish<Q, L>(acc[j], d, ux, uy, uz);
+            if (store >> (j + 1) & 1u) {
+                step_store<ST>(a.post, zoff + xy + (uint32_t)(j * a.nx), d.v.x, ux.v.x, uy.v.x, uz.v.x, scale, a.seed);
+                if constexpr (AMAX) track_amax(amax, d.v.x, ux.v.x, uy.v.x, uz.v.x);
+            }
+            if (store >> (j + NP + 1) & 1u) {
+                step_store<ST>(a.post, zoff + xy + (uint32_t)((j + NP) * a.nx), d.v.y, ux.v.y, uy.v.y, uz.v.y, scale, a.seed);
+                if constexpr (AMAX) track_amax(amax, d.v.y, ux.v.y, uy.v.y, uz.v.y);
+            }
+        }
+        // plane p: the links from the plane below and from its own
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            L v[Q];
+            links_of<Q, 0>([&](auto kc) { v[decltype(kc)::value] = brings(kc, j); });
+            if (walls) {
+                links_of<Q, 1>([&](auto kc) {
+                    constexpr int K = decltype(kc)::value;
+                    up[j][K] = or_wall(kc, Below{}, j, up[j][K], out[j][inv_dir(K)]);
+                });
+                links_of<Q, 0>([&](auto kc) {
+                    constexpr int K = decltype(kc)::value;
+                    v[K] = or_wall(kc, Here{}, j, v[K], out[j][inv_dir(K)]);
+                });
+            }
+            acc[j].S[0] = out[j][0];
+            links_of<Q, 1>([&](auto kc) { acc[j].template add<Q, decltype(kc)::value>(up[j][decltype(kc)::value]); });
+            links_of<Q, 0>([&](auto kc) { acc[j].template add<Q, decltype(kc)::value>(v[decltype(kc)::value]); });
+            links_of<Q, 1>([&](auto kc) {
+                constexpr int K = decltype(kc)::value;
+                up[j][K] = brings(kc, j);
+                own[j][K] = out[j][K];
+            });
+        }
+        slot = next;
+    }
+}
+
 // Rows per strip, and resident blocks the register budget is sized for. Four rows
 // form six rows' moments for four, two rows four for two, but two leave
 // registers for more warps.
-template <typename E, int V> struct StripShape;
-template <> struct StripShape<float, 0> { static constexpr int R = 2, MINB = 4; };
-template <> struct StripShape<float, 1> { static constexpr int R = 4, MINB = 3; };
-template <> struct StripShape<float, 2> { static constexpr int R = 4, MINB = 2; };
-template <int V> struct StripShape<double, V> { static constexpr int R = 2, MINB = 2; };
+template <int Q, int ST, int V> struct StripShape;
+template <int Q> struct StripShape<Q, ST_F32, 0> { static constexpr int R = 2, MINB = 4; };
+template <int Q> struct StripShape<Q, ST_F32, 1> { static constexpr int R = 4, MINB = 3; };
+template <int Q> struct StripShape<Q, ST_F32, 2> { static constexpr int R = 4, MINB = 2; };
+template <int Q, int V> struct StripShape<Q, ST_F64, V> { static constexpr int R = 2, MINB = 2; };
+// Link by link, two rows fill the registers: D3Q27 spills 200 bytes at 4 blocks
+// (256^3 BF16 225 us per step, 206 at 3) and 90 with four rows.
+template <int Q, int V> struct LinkShape;
+template <int Q> struct LinkShape<Q, 0> { static constexpr int R = 2, MINB = Q == 19 ? 4 : 3; };
+template <int Q> struct LinkShape<Q, 1> { static constexpr int R = 2, MINB = Q == 19 ? 3 : 2; };
+template <int Q> struct LinkShape<Q, 2> { static constexpr int R = 4, MINB = 2; };
+template <int Q, int V> struct StripShape<Q, ST_F16S, V> : LinkShape<Q, V> {};
+template <int Q, int V> struct StripShape<Q, ST_BF16S, V> : LinkShape<Q, V> {};
 constexpr int STRIP_SHAPES = 3;  // FP32-arithmetic formats; FP64 has one
 
 }  // namespace col

@@ -1,5 +1,6 @@
-// Equilibria of a node link by link, for the D2Q9, BGK and Zou-He kernels (the 3D
-// step kernels sum them axis by axis: moments.cuh).
+// Equilibria of a node link by link, for the D2Q9, BGK and Zou-He kernels and for
+// 16-bit boxes (links.cuh); the 3D kernels of FP32 and FP64 boxes sum them axis by
+// axis (moments.cuh).
 //
 // Eq. (feq) with c_s^2 = 1/3, written as the deviation from the rest weight
 // and divided by the weight w_k:

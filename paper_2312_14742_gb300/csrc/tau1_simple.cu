@@ -3,10 +3,11 @@
 // The plain form of Algorithm "Tau1" (pull, AB layout) with the halfway
 // bounce-back of Algorithm "Complete Tau1 ... halfway bounce-back": the node
 // reads every source's record, forms its moments and takes the sums of
-// moments.cuh; wall links add the node's own equilibria. It serves any box
+// moments.cuh, or of links.cuh; wall links bring the node's own equilibria. It serves any box
 // shape and every storage format and is the cross-check of the tiled kernel,
 // which evaluates the same functions in the same order: both give the same bits.
 #include "kernels.h"
+#include "links.cuh"
 #include "moments.cuh"
 
 namespace lbm {
@@ -17,37 +18,47 @@ __global__ void __launch_bounds__(256) tau1_simple_kernel(StepArgs a)
     using T = typename Storage<ST>::ctype;
     const int64_t n = (int64_t)a.nx * a.ny * a.nz;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const Scales sc(a.dscale);
-    const Terms<ST> t(a, sc);
     if (i >= n) return;
-    const Rec<T> c0 = record<ST>(a.pre, (uint32_t)i);
-    if (isnan(c0.d)) return;  // solid node
+    const Scales sc(a.dscale);
+    T d0, ux0, uy0, uz0;
+    Storage<ST>::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
+    if (isnan(d0)) return;  // solid node
     const int x = (int)(i % a.nx);
     const int y = (int)((i / a.nx) % a.ny);
     const int z = (int)(i / ((int64_t)a.nx * a.ny));
-    const Moments<T> own = moments_of_record<ST>(c0, t);
-    uint32_t wall = 0;
-    T sums[4];
-    gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
+    auto load = [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
         constexpr int K = decltype(kc)::value;
         int sx = x - cvel(K, 0), sy = y - cvel(K, 1), sz = z - cvel(K, 2);
         bool inside = true;
         if (sx < 0 || sx >= a.nx) { if (a.periodic[0]) sx = sx < 0 ? sx + a.nx : sx - a.nx; else inside = false; }
         if (sy < 0 || sy >= a.ny) { if (a.periodic[1]) sy = sy < 0 ? sy + a.ny : sy - a.ny; else inside = false; }
         if (sz < 0 || sz >= a.nz) { if (a.periodic[2]) sz = sz < 0 ? sz + a.nz : sz - a.nz; else inside = false; }
-        Rec<T> c{T(NAN), T(0), T(0), T(0)};
+        d = T(NAN);
+        ux = uy = uz = T(0);
         if (inside) {
             const int64_t s = (int64_t)sx + (int64_t)a.nx * ((int64_t)sy + (int64_t)a.ny * sz);
-            c = record<ST>(a.pre, (uint32_t)s);
+            Storage<ST>::load(a.pre, (uint32_t)s, sc.inv, d, ux, uy, uz);
         }
-        solid = isnan(c.d);
-        if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
-        return c;
-    }, sums);
-    add_bounce<Q, T>(own, wall, sums);
-
+        solid = isnan(d);
+    };
     T d, ux, uy, uz;
-    node_state<Q, T>(sums, d, ux, uy, uz);
+    if constexpr (by_links(ST)) {
+        gather_links<Q, T>(a, d0, ux0, uy0, uz0, load, d, ux, uy, uz);
+    } else {
+        const Terms<ST> t(a);
+        const Moments<T> own = moments_of<ST, T>({d0, ux0, uy0, uz0}, t, false);
+        uint32_t wall = 0;
+        T sums[4];
+        gather_sums<Q, ST>(t, own, [&](auto kc, bool& solid) {
+            constexpr int K = decltype(kc)::value;
+            Rec<T> c;
+            load(kc, solid, c.d, c.ux, c.uy, c.uz);
+            if (solid) wall |= 1u << nbit(-cvel(K, 0), -cvel(K, 1), -cvel(K, 2));
+            return c;
+        }, sums);
+        add_bounce<Q, T>(own, wall, sums);
+        node_state<Q, T>(sums, d, ux, uy, uz);
+    }
     step_store<ST>(a.post, (uint32_t)i, d, ux, uy, uz, sc.s, a.seed);
 }
 
