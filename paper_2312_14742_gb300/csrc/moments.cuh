@@ -45,23 +45,29 @@ template <typename T> struct IsFp64<T, std::void_t<typename T::elem>> : std::is_
 // but 1.5 u has at most one bit more than u, so that rounding it, with the
 // constant 1.5 g added, errs to the same side step after step: a channel's
 // momentum was 1e-6 off after 100 steps. These V have full mantissas, and u V
-// rounds as any number does: 1.3e-7. The two products hold to 9e-12 in FP32
-// (constants with 24 bits) and to 4e-21 in FP64.
+// rounds as any number does: 1.3e-7. The two products hold to 5e-13 in FP32
+// (constants with 24 bits) and to 2e-23 in FP64.
+// A = drho - r vv / 3 takes back the trace of the quadratic terms, and what it
+// leaves is lost or gained by every node in every step: a third rounded to 24 bits
+// cost 4.5e-8 u.u of density a step. So R / 3 has 24 bits too, and r / 3 is
+// rounded from drho by itself.
 template <typename T> struct Scale {
-    static constexpr double V = IsFp64<T>::value ? 1.5487772433133968 : 1.5476521253585815;
-    static constexpr double R = IsFp64<T>::value ? 1.8760076119698332 : 1.8787362575531006;
-    static constexpr double L = IsFp64<T>::value ? 1.0325181622089312 : 1.0317680835723877;
+    static constexpr double V = IsFp64<T>::value ? 1.544922908228737 : 1.5488158464431763;
+    static constexpr double R = IsFp64<T>::value ? 1.885379965393459 : 1.8759140968322754;
+    static constexpr double L = IsFp64<T>::value ? 1.0299486054858247 : 1.0325438976287842;
+    static constexpr double R3 = R / 3.0;
+    static_assert(3.0 * R3 == R && (IsFp64<T>::value || (double)(float)R3 == R3), "a third without rounding");
 };
 
 template <typename T> struct Moments {
     T A, r, vx, vy, vz;
 };
 
-// From d = drho, r and v (a solid node: d = r = 0).
-template <typename T> __device__ __forceinline__ Moments<T> moments_from(T d, T r, T vx, T vy, T vz)
+// What a node's density leaves after the trace, from d = drho.
+template <typename T> __device__ __forceinline__ T less_trace(T d, T vx, T vy, T vz)
 {
     const T vv = fma(vz, vz, fma(vy, vy, vx * vx));
-    return {fma(T(-1.0 / 3.0) * r, vv, d), r, vx, vy, vz};
+    return fma(fma(T(-Scale<T>::R3), d, T(-Scale<T>::R3)), vv, d);
 }
 
 // A product as one fused operation (+0 for a zero product of either sign): its
@@ -105,11 +111,8 @@ template <int ST> __device__ __forceinline__ Rec<typename Storage<ST>::ctype> re
 template <int ST, typename T>
 __device__ __forceinline__ Moments<T> moments_of(const Rec<T>& c, const Terms<ST>& t, bool solid)
 {
-    return moments_from<T>(solid ? T(0) : c.d, solid ? T(0) : t.r(c.d), t.vx(c.ux), t.vy(c.uy), t.vz(c.uz));
-}
-template <int ST, typename T> __device__ __forceinline__ Moments<T> moments_of_record(const Rec<T>& c, const Terms<ST>& t)
-{
-    return moments_of<ST, T>(c, t, isnan(c.d));  // drho NaN: a solid node
+    const T vx = t.vx(c.ux), vy = t.vy(c.uy), vz = t.vz(c.uz), A = less_trace<T>(c.d, vx, vy, vz);
+    return {solid ? T(0) : A, solid ? T(0) : t.r(c.d), vx, vy, vz};
 }
 
 // c.v for a constant direction c (axis order x, y, z).
@@ -360,14 +363,14 @@ __device__ __forceinline__ void node_state(const T (&s)[4], T& d, T& ux, T& uy, 
 template <int MIRROR, int ST, typename L, typename E>
 __device__ __forceinline__ Moments<L> pair_moments(const Rec<E>& a, const Rec<E>& b, const Terms<ST>& t, bool sA, bool sB)
 {
-    const L d = L(sA ? E(0) : a.d, sB ? E(0) : b.d);
     const L r = L(sA ? E(0) : t.r(a.d), sB ? E(0) : t.r(b.d));
     L vx = L(t.vx(a.ux), t.vx(b.ux));
     L vy = L(t.vy(a.uy), t.vy(b.uy));
     const L vz = L(t.vz(a.uz), t.vz(b.uz));
     if constexpr (MIRROR == 1) vx.v.y = -vx.v.y;
     if constexpr (MIRROR == 2) vy.v.y = -vy.v.y;
-    return moments_from<L>(d, r, vx, vy, vz);
+    const L A = less_trace<L>(L(a.d, b.d), vx, vy, vz);
+    return {L(sA ? E(0) : A.v.x, sB ? E(0) : A.v.y), r, vx, vy, vz};
 }
 
 // Direction index of a velocity (-1: none).
