@@ -39,6 +39,8 @@ struct lbm_tau1 {
     float scale_host[8] = {};           // staging for scale copies
     int kernel = LBM_KERNEL_SIMPLE;
     int variant = 0;            // tile-shape variant of the tiled kernel
+    int sms = 0;                // SMs of the handle's device
+    StripPlan plan{};           // tiled kernel: strips of the variant
     bool sparse = false;        // fluid-list layout: buf holds nf records
     int64_t nf = 0;             // sparse: fluid nodes in the list
     int* pos = nullptr;         // sparse: box node of each list entry
@@ -381,6 +383,14 @@ lbm_status build_compact(lbm_tau1* h)
     return LBM_OK;
 }
 
+// Strips of a variant of the tiled kernel (not of D2Q9 or the compact layout).
+StripPlan plan_of(const lbm_tau1* h, int variant)
+{
+    const lbm_tau1_config& c = h->cfg;
+    if (c.q == LBM_D2Q9 || h->kernel != LBM_KERNEL_TILED) return {};
+    return strip_plan(c.q, c.storage, variant, c.nx, c.ny, c.nz, c.periodic[0] ? 1 : 0, h->sms);
+}
+
 // Kernel launches of one step of the main kernel(s).
 int step_launches(const lbm_tau1* h)
 {
@@ -388,7 +398,7 @@ int step_launches(const lbm_tau1* h)
     return (h->n_ctiles > 0 ? 1 : 0) + (h->n_cnodes > 0 ? 1 : 0);
 }
 
-cudaError_t launch_kernel(const lbm_tau1* h, int variant, const StepArgs& a)
+cudaError_t launch_kernel(const lbm_tau1* h, const StripPlan& plan, const StepArgs& a)
 {
     if (h->cfg.q == LBM_D2Q9) return launch_tau1_2d(h->kernel == LBM_KERNEL_SIMPLE, h->cfg.storage, a, h->stream);
     if (h->compact) {
@@ -404,7 +414,7 @@ cudaError_t launch_kernel(const lbm_tau1* h, int variant, const StepArgs& a)
         return e;
     }
     if (h->sparse) return launch_tau1_sparse(h->cfg.q, h->cfg.storage, a, (int)h->nf, h->nbr, h->stream);
-    if (h->kernel == LBM_KERNEL_TILED) return launch_tau1_tiled(h->cfg.q, h->cfg.storage, variant, a, h->stream);
+    if (h->kernel == LBM_KERNEL_TILED) return launch_tau1_tiled(h->cfg.q, h->cfg.storage, plan, a, h->stream);
     return launch_tau1_simple(h->cfg.q, h->cfg.storage, a, h->stream);
 }
 
@@ -421,7 +431,7 @@ lbm_status launch_step(lbm_tau1* h)
         ++h->step;
         return LBM_OK;
     }
-    cudaError_t e = launch_kernel(h, h->variant, a);
+    cudaError_t e = launch_kernel(h, h->plan, a);
     if (e != cudaSuccess) return cuda_fail(h, e, "tau1 step launch");
     h->launches += step_launches(h);
     if (h->p_axis >= 0) {
@@ -447,11 +457,11 @@ lbm_status time_compact(lbm_tau1* h, int trials, cudaEvent_t e0, cudaEvent_t e1,
 {
     StepArgs a;
     fill_args(h, a);
-    cudaError_t e = launch_kernel(h, 0, a);
+    cudaError_t e = launch_kernel(h, h->plan, a);
     h->launches += step_launches(h);
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
     for (int t = 0; t < trials && e == cudaSuccess; ++t) {
-        e = launch_kernel(h, 0, a);
+        e = launch_kernel(h, h->plan, a);
         h->launches += step_launches(h);
     }
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
@@ -574,7 +584,10 @@ lbm_status lbm_tau1_create(const lbm_tau1_config* cfg, lbm_tau1** out)
         delete h;
         return fail(nullptr, LBM_EINVAL, "create: tiled kernel not available for this lattice/storage");
     }
-    cudaError_t e = cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) h->plan = plan_of(h, h->variant);
     h->bgk = cfg->scheme == LBM_SCHEME_BGK;
     // dense: two copies of the box; sparse: allocated by set_geometry (nf records)
     // (compact: one more record, the solid sentinel of the node-list kernel)
@@ -830,6 +843,7 @@ lbm_status lbm_tau1_set_variant(lbm_tau1* h, int32_t variant)
     if (!h) return fail(nullptr, LBM_EINVAL, "set_variant: NULL handle");
     if (variant < 0 || variant >= variant_count(h)) return fail(h, LBM_EINVAL, "set_variant: no such variant");
     h->variant = variant;
+    h->plan = plan_of(h, variant);
     return (h->compact && h->has_geometry) ? build_compact(h) : LBM_OK;
 }
 
@@ -897,6 +911,7 @@ lbm_status lbm_tau1_autotune(lbm_tau1* h, int32_t trials, int32_t* chosen, float
     double cached_ms = 0;
     if (tune_cache_lookup(key, &cached, &cached_ms) && cached >= 0 && cached < variant_count(h)) {
         h->variant = cached;
+        h->plan = plan_of(h, cached);
         if (chosen) *chosen = cached;
         if (ms_per_step) *ms_per_step = (float)cached_ms;
         return LBM_OK;
@@ -913,11 +928,12 @@ lbm_status lbm_tau1_autotune(lbm_tau1* h, int32_t trials, int32_t* chosen, float
     int best = h->variant;
     float best_ms = 0.f;
     for (int v = 0; v < nv && e == cudaSuccess; ++v) {
-        e = launch_kernel(h, v, a);  // warm-up (and first-use set-up)
+        const StripPlan plan = plan_of(h, v);
+        e = launch_kernel(h, plan, a);  // warm-up (and first-use set-up)
         ++h->launches;
         if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
         for (int t = 0; t < trials && e == cudaSuccess; ++t) {
-            e = launch_kernel(h, v, a);
+            e = launch_kernel(h, plan, a);
             ++h->launches;
         }
         if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
@@ -931,6 +947,7 @@ lbm_status lbm_tau1_autotune(lbm_tau1* h, int32_t trials, int32_t* chosen, float
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune: trial");
     h->variant = best;
+    h->plan = plan_of(h, best);
     if (chosen) *chosen = best;
     if (ms_per_step) *ms_per_step = best_ms;
     tune_cache_store(key, best, best_ms);

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(Cfg<Q, ST, R>::NT, 4 * MINB / Cfg<Q, ST, R>::W
         const int local = uniform(it - begin[lo]);
         const uint32_t c = (uint32_t)uniform((int)D.cur);
         const StepArgs a = uniform_args(D, c);
-        const int nstrips = uniform(D.nstrips), z0 = local / nstrips * chunk, z1 = min(a.nz, z0 + chunk);
+        const int nstrips = uniform(D.nstrips), z0 = local / nstrips * chunk, z1 = a.nz - z0 < chunk ? a.nz : z0 + chunk;
         const Place pl = place_of_strip<R>(a, local % nstrips);
         unsigned char* const mine = smem + warp * Cfg<Q, ST, R>::WARP;
         [[maybe_unused]] float amax[4] = {0.f, 0.f, 0.f, 0.f};
@@ -232,8 +232,6 @@ cudaError_t batch_prepare(int q, int storage, int variant, int* grid, int* rows)
     *rows = r;
     return e;
 }
-
-long long batch_strips(int nx, int ny, int periodic, int rows) { return strips_of(nx, ny, periodic, rows); }
 
 cudaError_t launch_tau1_batch(int q, int storage, int variant, BatchTable* T, int grid, cudaStream_t s)
 {

@@ -34,9 +34,8 @@ struct BatchTable {
 };
 
 // Persistent grid size (blocks of 4 warps, a work item per warp) and rows per
-// strip of a kernel variant; strips per plane of a box.
+// strip of a kernel variant.
 cudaError_t batch_prepare(int q, int storage, int variant, int* grid, int* rows);
-long long batch_strips(int nx, int ny, int periodic, int rows);
 cudaError_t launch_tau1_batch(int q, int storage, int variant, BatchTable* T, int grid, cudaStream_t s);
 
 }  // namespace lbm

@@ -141,7 +141,7 @@ cudaError_t stage_done(Stage* s, cudaStream_t stream)
 }
 
 // Work items of a box for a chunk height.
-int box_items(const Slot& s, int chunk) { return s.nstrips * ((s.cfg.nz + chunk - 1) / chunk); }
+int64_t box_items(const Slot& s, int chunk) { return (int64_t)s.nstrips * (((int64_t)s.cfg.nz + chunk - 1) / chunk); }
 
 // Rebuilds the live list and item offsets and queues their upload. The chunk
 // is the one with the least (waves of items over the persistent grid's warps) x (planes
@@ -417,7 +417,7 @@ lbm_status lbm_tau1_batch_admit(lbm_tau1_batch* b, const lbm_tau1_config* cfg, c
     }
     rec.buf[0] = s.buf[0];
     rec.buf[1] = s.buf[1];
-    rec.nstrips = (int)batch_strips(cfg->nx, cfg->ny, rec.a.periodic[0], b->rows);
+    rec.nstrips = (int)strips_of(cfg->nx, cfg->ny, rec.a.periodic[0], b->rows);
     rec.cur = 0;
     rec.step = 0;
     for (int c = 0; c < 2; ++c)

@@ -284,7 +284,7 @@ CompactTiles compact_tiles(int q, int storage, int variant)
     t.shape = nr == 1 ? 0 : ((v < 2) != by_links(storage) ? 1 : 0);
     t.zchunk = variant < nr ? 24 : 32;
     t.h = v == 1 ? 16 : (v == 3 ? 12 : 8);
-    t.rows = tau1_strip_rows(q, storage, t.shape);
+    t.rows = strip_shape(q, storage, t.shape).rows;
     return t;
 }
 

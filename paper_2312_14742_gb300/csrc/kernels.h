@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "strip_plan.h"
 
 namespace lbm {
 
@@ -13,7 +14,8 @@ namespace lbm {
 cudaError_t launch_tau1_simple(int q, int storage, const StepArgs& a, cudaStream_t s);
 // Tiled kernel (tau1_strip.cu): variant v is shape choice v % R, R =
 // tau1_tile_shapes (0: by the box), with z chunks by the box, of 32, 16 or 48 planes (v / R).
-cudaError_t launch_tau1_tiled(int q, int storage, int variant, const StepArgs& a, cudaStream_t s);
+// Its plan, from strip_plan(), holds for a box and variant.
+cudaError_t launch_tau1_tiled(int q, int storage, const StripPlan& plan, const StepArgs& a, cudaStream_t s);
 bool tau1_tiled_supported(int q, int storage, int64_t n);
 int tau1_tiled_variants(int q, int storage);
 int tau1_tile_shapes(int storage);
@@ -23,8 +25,6 @@ int tau1_tile_shapes(int storage);
 // chunk of zchunk planes. An owned column has its neighbours in the next lanes.
 // after_list: the last launch on s is launch_tau1_list() of the same step.
 constexpr int STRIP_ITEM = 33;
-constexpr int STRIP_WARPS = 4;  // warps per block of the dense and batched kernels, a strip each
-int tau1_strip_rows(int q, int storage, int shape);
 cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
                                    int count, bool after_list, cudaStream_t s);
 // Self-test (selftest.cu): one warp waits, bounded, on an mbarrier phase

@@ -39,6 +39,7 @@
 #include "mbarrier.cuh"
 #include "moments.cuh"
 #include "pack2.cuh"
+#include "strip_plan.h"
 
 namespace lbm {
 
@@ -162,20 +163,12 @@ template <int R> __device__ __forceinline__ Place place_of_slot(const StepArgs& 
 // Strip i of a box: 30 slots of the sequence, the first and last lane hold the
 // ones before and after. A periodic box of 32 columns takes a lane per column
 // and rotates them.
-__host__ __device__ __forceinline__ bool rotates(int nx, int periodic) { return nx == 32 && periodic; }
 template <int R> __device__ __forceinline__ Place place_of_strip(const StepArgs& a, int i)
 {
     const int lane = threadIdx.x & 31;
-    if (rotates(a.nx, a.periodic[0])) return {lane, i * R, true, (lane + 31) & 31, (lane + 1) & 31};
+    if (strip_rotates(a.nx, a.periodic[0])) return {lane, i * R, true, (lane + 31) & 31, (lane + 1) & 31};
     return place_of_slot<R>(a, 30u * (uint32_t)i + (uint32_t)lane, lane >= 1 && lane <= 30);
 }
-// Strips of a plane of nx x ny nodes.
-__host__ __device__ __forceinline__ long long strips_of(int nx, int ny, int periodic, int R)
-{
-    const long long rows = ((long long)ny + R - 1) / R;
-    return rotates(nx, periodic) ? rows : (rows * ((long long)nx + 2) - 2 + 29) / 30;
-}
-
 // The planes of a strip as they pass through a warp's shared memory: R + 2 rows
 // of 32 records, a slot per plane, each lane's cells copied by the lane itself.
 // A cell beyond a non-periodic face holds a wall's record.
@@ -601,7 +594,6 @@ template <int Q> struct LinkShape<Q, 1> { static constexpr int R = 2, MINB = Q =
 template <int Q> struct LinkShape<Q, 2> { static constexpr int R = 4, MINB = 2; };
 template <int Q, int V> struct StripShape<Q, ST_F16S, V> : LinkShape<Q, V> {};
 template <int Q, int V> struct StripShape<Q, ST_BF16S, V> : LinkShape<Q, V> {};
-constexpr int STRIP_SHAPES = 3;  // FP32-arithmetic formats; FP64 has one
 
 }  // namespace col
 

@@ -1,0 +1,58 @@
+"""The strips that a box is cut into (csrc/strip_plan.h), as plain C++ on the host."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2312_14742_gb300", "csrc")
+
+CPP = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "strip_plan.h"
+int main(int argc, char** argv)
+{
+    int a[8];
+    while (std::scanf("%d %d %d %d %d %d %d %d", a, a + 1, a + 2, a + 3, a + 4, a + 5, a + 6, a + 7) == 8) {
+        const lbm::StripPlan p = lbm::strip_plan(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7]);
+        const lbm::StripShapeCost s = lbm::strip_shape(a[0], a[1], p.shape);
+        const long long strips = lbm::strips_of(a[3], a[4], a[6], s.rows);
+        std::printf("%d %d %d %lld %lld\n", p.shape, p.chunk, s.rows, strips,
+                    strips * (((long long)a[5] + p.chunk - 1) / p.chunk));
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text(CPP)
+    exe = str(d / "plan")
+    # signed overflow ends the program
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-ftrapv", "-I", CSRC, str(d / "plan.cpp"), "-o", exe])
+
+    def ask(boxes):
+        text = "\n".join(" ".join(map(str, b)) for b in boxes)
+        r = subprocess.run([exe], input=text, capture_output=True, text=True, timeout=60)
+        assert r.returncode == 0
+        got = [tuple(map(int, l.split())) for l in r.stdout.splitlines()]
+        assert len(got) == len(boxes)
+        return got
+
+    return ask
+
+
+def test_boxes_of_every_shape(plans):
+    """Every variant gives a chunk of 1 .. nz planes and a number of strips that fits
+    an int, for boxes of up to 2^31 - 2 nodes along any axis."""
+    big = (1 << 31) - 2
+    dims = [(1, 1, 1), (32, 1, 1), (256, 256, 256), (1, 1, big), (1, 1, (1 << 30) + 10), (1, big, 1), (big, 1, 1),
+            (2, 2, (1 << 29) - 1), (1, 1 << 15, (1 << 16) - 1), (46340, 46340, 1)]
+    boxes = [(q, st, v, nx, ny, nz, per, 152) for nx, ny, nz in dims for q in (19, 27) for st in range(4)
+             for v in range(4 if st == 0 else 16) for per in (0, 1)]
+    for box, (shape, chunk, rows, strips, items) in zip(boxes, plans(boxes)):
+        nx, ny, nz = box[3:6]
+        assert 0 <= shape < (1 if box[1] == 0 else 3) and 1 <= chunk <= nz, box
+        assert 30 * strips * rows >= nx * ny or nx == 32, box
+        assert 0 < items < (1 << 31) - 8, box
