@@ -245,9 +245,9 @@ lbm_status lbm_tau1_set_variant(lbm_tau1* h, int32_t variant);
 lbm_status lbm_tau1_autotune(lbm_tau1* h, int32_t trials, int32_t* chosen, float* ms_per_step);
 
 /* Autotune cache for the whole process: path of a JSON file of chosen
- * variants keyed by device name, lattice, storage, layout, size bucket
- * (ceil log2 of nx*ny*nz) and whether the box has full tiles. With a cache
- * set, lbm_tau1_autotune first looks its key up and, when found, selects that
+ * variants keyed by device name, lattice, storage, layout, the library's
+ * kernels and the box (entries of a library whose variants meant other kernels
+ * are kept but not used). With a cache set, lbm_tau1_autotune first looks its key up and, when found, selects that
  * variant without timing (returning the stored ms per step); otherwise it
  * times the variants and writes its choice to the file. NULL or "" turns the
  * cache off (the default). The file is read and rewritten on each use. */

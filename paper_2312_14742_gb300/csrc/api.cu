@@ -250,8 +250,10 @@ lbm_status bgk_from_state(lbm_tau1* h)
 }
 
 // Autotune cache key: device, lattice, storage, layout, size bucket
-// (ceil log2 of the node count) and whether every tile is full (the staged
-// kernel's condition), e.g. "NVIDIA GB300/D3Q19/F32/dense/n2^24/full".
+// (ceil log2 of the node count), whether nx is a multiple of 32 and ny of 16, and
+// then what decides whether a variant's time holds: the kernels that the variant
+// numbers mean (changed with that meaning) and the box that its strips are cut
+// from, e.g. "NVIDIA GB300/D3Q19/F32/dense/n2^24/full/strips/256x256x256/x".
 std::string tune_key(const lbm_tau1* h)
 {
     int dev = 0;
@@ -263,8 +265,9 @@ std::string tune_key(const lbm_tau1* h)
     while (((int64_t)1 << lg) < h->n) ++lg;
     const bool full = h->cfg.nx % 32 == 0 && h->cfg.ny % 16 == 0;
     char buf[256];
-    std::snprintf(buf, sizeof(buf), "%s/D3Q%d/%s/%s/n2^%d/%s", name.c_str(), h->cfg.q, st[h->cfg.storage],
-                  h->sparse ? "sparse" : "dense", lg, full ? "full" : "ragged");
+    std::snprintf(buf, sizeof(buf), "%.120s/D3Q%d/%s/%s/n2^%d/%s/strips/%dx%dx%d%s", name.c_str(), h->cfg.q,
+                  st[h->cfg.storage], h->sparse ? "sparse" : "dense", lg, full ? "full" : "ragged", h->cfg.nx, h->cfg.ny,
+                  h->cfg.nz, h->cfg.periodic[0] ? "/x" : "");
     return buf;
 }
 

@@ -1,6 +1,5 @@
-// Autotune cache: the tile-shape variant chosen for a (device, lattice,
-// storage, layout, size bucket, tile fit) key, kept in a JSON file so that
-// later handles skip the timing.
+// Autotune cache: the variant chosen for a (device, lattice, storage, layout,
+// kernels, box) key, kept in a JSON file so that later handles skip the timing.
 //
 // File format (written and read here only):
 //   {"version": 1, "entries": {
