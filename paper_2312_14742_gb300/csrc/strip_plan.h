@@ -23,22 +23,28 @@ constexpr int64_t strips_of(int nx, int ny, int periodic, int rows_per_strip)
 constexpr int STRIP_SHAPES = 3;  // per lattice and format; FP64 has one
 
 // A shape of strips: its rows, the resident blocks per SM that its registers are
-// sized for, and the time of a plane with 0 .. 4 blocks on an SM.
+// sized for, and the time of a plane with 0 .. 4 blocks on an SM, and in many waves
+// where that is not the last of them.
 struct StripShapeCost {
     int rows, minb;
-    double plane[5];
+    double plane[5], many = 0;
 };
 
 // Storage 0 FP64, 1 FP32, 2 and 3 the 16-bit formats (lbm_storage). The times of a
-// plane, up to a factor, are fitted to sweeps of shape and chunk over 11 boxes.
-// Measured, in us, with four rows and two: D3Q19 FP32 96^3 16.6 and 14.6,
-// 250 x 130 x 90 34.7 and 33.0, 128^3 24.8 and 26.3, 384^3 408 and 428.
+// plane, up to a factor, are fitted to sweeps of shape and chunk over 18 boxes.
+// Measured in FP32, in us, with two rows and four: D3Q19 256^3 138 and 135,
+// 512 x 256 x 128 138 and 133, 384^3 416 and 400, 128^3 26.7 and 25.3, but
+// 250 x 130 x 90 34.5 and 37.2, 96^3 14.4 and 16.4; D3Q27 256^3 147 and 163, 320^3 267
+// and 296, 250 x 130 x 90 37.0 and 45, 200^3 92.5 and 90.4, 96 x 256 x 128 without
+// walls 34.7 and 28.8. On 11 boxes left out of the fit the default is the faster of
+// the two, or within 2% of it.
 constexpr StripShapeCost strip_shape(int q, int storage, int v)
 {
     if (storage == 0) return {2, 2, {0, 1.2, 2.0, 0, 0}};
     if (storage == 1)
-        return v == 0 ? StripShapeCost{2, 4, {0, 0.95, 1.3, 1.7, 2.1}}
-                      : (v == 1 ? StripShapeCost{4, 3, {0, 1.6, 2.3, 3.0, 0}} : StripShapeCost{4, 2, {0, 1.6, 2.3, 0, 0}});
+        return v == 0 ? StripShapeCost{2, 4, {0, 0.95, 1.3, 1.7, 2.1}, q == 19 ? 2.2 : 2.1}
+                      : (v == 1 ? StripShapeCost{4, 3, {0, 1.6, 2.3, 3.0, 0}, q == 19 ? 3.0 : 3.24}
+                                : StripShapeCost{4, 2, {0, 1.6, 2.3, 0, 0}});
     if (q == 19)
         return v == 0 ? StripShapeCost{2, 4, {0, 0.87, 1.2, 1.56, 1.93}}
                       : (v == 1 ? StripShapeCost{2, 3, {0, 0.87, 1.2, 1.56, 0}} : StripShapeCost{4, 2, {0, 1.6, 2.3, 0, 0}});
@@ -56,7 +62,8 @@ inline double strip_cost(int64_t nz, int64_t strips, int64_t chunk, int sms, con
     const int64_t blocks = (strips * ((nz + chunk - 1) / chunk) + STRIP_WARPS - 1) / STRIP_WARPS;
     const double planes = (double)chunk + 4, waves = (double)blocks / ((double)sms * s.minb);
     if (waves <= 1) return planes * 1.15 * s.plane[(blocks + sms - 1) / sms];
-    return planes * s.plane[s.minb] * (waves <= 2.5 ? 1.15 * std::ceil(waves) : waves + 0.4);
+    if (waves <= 2.5) return planes * s.plane[s.minb] * 1.15 * std::ceil(waves);
+    return planes * (s.many > 0 ? s.many : s.plane[s.minb]) * (waves + 0.4);
 }
 
 struct StripPlan {

@@ -56,3 +56,14 @@ def test_boxes_of_every_shape(plans):
         assert 0 <= shape < (1 if box[1] == 0 else 3) and 1 <= chunk <= nz, box
         assert 30 * strips * rows >= nx * ny or nx == 32, box
         assert 0 < items < (1 << 31) - 8, box
+
+
+def test_fp32_boxes_take_the_faster_shape(plans):
+    """By default two rows or four, whichever was measured the faster by 2% or more."""
+    two, four = 2, 4
+    boxes = [(19, (256, 256, 256), four), (19, (512, 256, 128), four), (19, (384, 384, 384), four),
+             (19, (128, 128, 128), four), (19, (250, 130, 90), two), (19, (96, 96, 96), two), (19, (161, 127, 101), two),
+             (27, (256, 256, 256), two), (27, (250, 130, 90), two), (27, (200, 200, 200), four),
+             (27, (96, 256, 128), four), (19, (100, 300, 120), four), (19, (160, 160, 160), four), (27, (320, 320, 320), two)]
+    got = plans([(q, 1, 0, *d, 1, 152) for q, d, _ in boxes])
+    assert [rows for _, _, rows, _, _ in got] == [rows for _, _, rows in boxes]
