@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12
         };
         T d, ux, uy, uz;
         if constexpr (by_links(ST)) {
-            gather_links<Q, T>(a, r[0].d, r[0].ux, r[0].uy, r[0].uz, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
+            gather_links<Q, false>(a, r[0].d, r[0].ux, r[0].uy, r[0].uz, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
                 const Rec<T>& c = fetch(kc, solid);
                 d = c.d;
                 ux = c.ux;

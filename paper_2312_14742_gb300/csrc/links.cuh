@@ -97,9 +97,10 @@ __device__ __forceinline__ void node_finish(const NodeAcc<T, Weights<Q>::NCLASS>
     uz = jz * r;
 }
 
-// One node gathered by one thread, own its record; load(k, solid, d, ux, uy, uz)
-// gives the record of the source x - c_k, or says that it is a wall.
-template <int Q, typename T, typename F>
+// One node gathered by one thread from its record and load(k, solid, d, ux, uy, uz),
+// which gives the record of the source x - c_k or says that it is a wall. SKIP:
+// a wall's record is not evaluated at all, where that pays for the branch.
+template <int Q, bool SKIP, typename T, typename F>
 __device__ __forceinline__ void gather_links(const StepArgs& a, T d0, T ux0, T uy0, T uz0, F&& load, T& d, T& ux, T& uy, T& uz)
 {
     const T gx = gcomp<T>(a, 0), gy = gcomp<T>(a, 1), gz = gcomp<T>(a, 2);
@@ -111,8 +112,11 @@ __device__ __forceinline__ void gather_links(const StepArgs& a, T d0, T ux0, T u
         T sd, sx, sy, sz;
         bool solid = false;
         load(kc, solid, sd, sx, sy, sz);
-        const NodeMoments<T> m = node_moments<T>(sd, sx, sy, sz, gx, gy, gz);
-        const T v = feq_scaled(m.A, m.H, dir_dot<K, T>(m.Px, m.Py, m.Pz));
+        T v = T(0);
+        if (!SKIP || !solid) {
+            const NodeMoments<T> m = node_moments<T>(sd, sx, sy, sz, gx, gy, gz);
+            v = feq_scaled(m.A, m.H, dir_dot<K, T>(m.Px, m.Py, m.Pz));
+        }
         // reflected population: own state in direction inv(k), p(inv k) = -p(k)
         const T b = feq_scaled(own.A, own.H, -dir_dot<K, T>(own.Px, own.Py, own.Pz));
         acc.template add<Q, K>(solid ? b : v);

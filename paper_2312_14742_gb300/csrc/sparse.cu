@@ -129,12 +129,16 @@ __global__ void __launch_bounds__(256) table_kernel(int nf, int nx, int ny, int 
 }
 
 // One Tau1 step of the fluid list: one thread per fluid node. D3Q19 hides the
-// latency of its gathers with warps (32 registers: 54.5 us for 1.8 M nodes, 61
+// latency of its gathers with warps (32 registers: 52.5 us for 1.8 M nodes, 61
 // with the registers the compiler would take); D3Q27 does better with more loads
-// in flight per thread (74 us against 95 at 40 registers). Summing link by link
-// took 55.5 and 82 us, and does in FP16, where the order of the links stays
-// (links.cuh), 61.6 and 82.
-constexpr int sparse_blocks(int q, int st) { return q == 19 && st == ST_F32 ? 8 : 0; }
+// in flight per thread (72 us against 95 at 40 registers). Summing link by link
+// took 55.5 and 82 us in FP32. The 16-bit formats do (links.cuh): BF16 51 and 70 us
+// with the indices first (59 and 93 each as it is used), FP16 54 and 81, where a
+// wall skips the scaling of a record (60 and 84 with the bounds of BF16).
+constexpr int sparse_blocks(int q, int st)
+{
+    return st == ST_F32 && q == 19 ? 8 : (st == ST_BF16S ? (q == 19 ? 6 : 4) : 0);
+}
 template <int Q, int ST>
 __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(StepArgs a, int nf, const int* __restrict__ nbr)
 {
@@ -142,24 +146,25 @@ __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf) return;
     const Scales sc(a.dscale);
+    // every index first: the records' loads then wait for none but their own
+    int src[Q];
+    static_for<1, Q>([&](auto kc) {
+        constexpr int K = decltype(kc)::value;
+        src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
+    });
     T d, ux, uy, uz;
     if constexpr (by_links(ST)) {
         T d0, ux0, uy0, uz0;
         Storage<ST>::load(a.pre, (uint32_t)i, sc.inv, d0, ux0, uy0, uz0);
-        gather_links<Q, T>(a, d0, ux0, uy0, uz0, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
+        gather_links<Q, ST == ST_F16S>(a, d0, ux0, uy0, uz0, [&](auto kc, bool& solid, T& d, T& ux, T& uy, T& uz) {
             constexpr int K = decltype(kc)::value;
-            const int j = __ldg(nbr + (int64_t)(K - 1) * nf + i);
+            const int j = src[K];
             solid = j < 0;
             d = ux = uy = uz = T(0);
             if (!solid) Storage<ST>::load(a.pre, (uint32_t)j, sc.inv, d, ux, uy, uz);
         }, d, ux, uy, uz);
     } else {
         const Terms<ST> t(a);
-        int src[Q];
-        static_for<1, Q>([&](auto kc) {
-            constexpr int K = decltype(kc)::value;
-            src[K] = __ldg(nbr + (int64_t)(K - 1) * nf + i);
-        });
         const Moments<T> own = moments_of<ST, T>(record<ST>(a.pre, (uint32_t)i), t, false);
         uint32_t wall = 0;
         T sums[4];

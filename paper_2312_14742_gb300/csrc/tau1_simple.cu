@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256) tau1_simple_kernel(StepArgs a)
     };
     T d, ux, uy, uz;
     if constexpr (by_links(ST)) {
-        gather_links<Q, T>(a, d0, ux0, uy0, uz0, load, d, ux, uy, uz);
+        gather_links<Q, false>(a, d0, ux0, uy0, uz0, load, d, ux, uy, uz);
     } else {
         const Terms<ST> t(a);
         const Moments<T> own = moments_of<ST, T>({d0, ux0, uy0, uz0}, t, false);
