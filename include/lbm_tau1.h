@@ -51,7 +51,7 @@ typedef enum {
     LBM_ENOMEM = 2,     /* device or host allocation failed */
     LBM_ECUDA = 3,      /* a CUDA call failed (message in last_error) */
     LBM_EDIVERGED = 4,  /* reduction saw a non-finite value or |u| > 0.3 */
-    LBM_ETIMEOUT = 5,   /* a bounded device wait (staged copy) ran out; the step results are unreliable */
+    LBM_ETIMEOUT = 5,   /* a bounded device wait ran out (the self-test; no step kernel waits) */
     LBM_EBUSY = 6,      /* no room (batch admission) */
     LBM_ESTATE = 7      /* call out of order (e.g. step before set_geometry) */
 } lbm_status;
@@ -171,8 +171,8 @@ lbm_status lbm_tau1_step(lbm_tau1* h, int64_t nsteps);
 lbm_status lbm_tau1_reduce(lbm_tau1* h, lbm_tau1_stats* out);
 
 /* Waits for all work queued on the handle's stream. Returns LBM_ETIMEOUT if
- * a staged (TMA) copy of a step kernel did not complete within its bounded
- * wait (about one second) since the last check; reduce reports the same. */
+ * a bounded device wait (about one second) ran out since the last check;
+ * reduce reports the same. No step kernel waits: only the self-test does. */
 lbm_status lbm_tau1_synchronize(lbm_tau1* h);
 
 /* Frees the handle and its device memory (after synchronising). NULL is a no-op. */
@@ -254,10 +254,9 @@ lbm_status lbm_tau1_autotune(lbm_tau1* h, int32_t trials, int32_t* chosen, float
 void lbm_tau1_set_tune_cache(const char* path);
 
 /* Self-test of the failure detection (no counterpart in the paper): queues
- * on the handle's stream one warp that waits, with the staged kernels'
- * bounded wait (about one second), on an mbarrier phase that nothing
- * completes, and counts the timeout in the handle's counter, as a staged
- * copy that never lands would. The next lbm_tau1_synchronize or
+ * on the handle's stream one warp that waits, bounded (about one second), on
+ * an mbarrier phase that nothing completes, and counts the timeout in the
+ * handle's counter. The next lbm_tau1_synchronize or
  * lbm_tau1_reduce then returns LBM_ETIMEOUT (and clears the count); nothing
  * faults and the context stays usable. For tests and health checks. */
 lbm_status lbm_tau1_selftest_timeout(lbm_tau1* h);
@@ -367,8 +366,8 @@ lbm_status lbm_tau1_batch_selftest_timeout(lbm_tau1_batch* b);
 
 /* Waits for the statistics queued by lbm_tau1_batch_stats_queue and fills
  * out[0..n-1] (n as queued). Returns LBM_EDIVERGED, with every out[] filled,
- * if any box diverged; LBM_ETIMEOUT if a staged-copy wait ran out in the
- * steps before the reductions; LBM_ESTATE if nothing was queued. */
+ * if any box diverged; LBM_ETIMEOUT after a self-test queued before
+ * them; LBM_ESTATE if nothing was queued. */
 lbm_status lbm_tau1_batch_stats_wait(lbm_tau1_batch* b, lbm_tau1_stats* out);
 
 /* State of a live box as doubles, as lbm_tau1_get_fields. */

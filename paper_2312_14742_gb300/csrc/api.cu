@@ -46,7 +46,8 @@ struct lbm_tau1 {
     int* pos = nullptr;         // sparse: box node of each list entry
     int* nbr = nullptr;         // sparse: neighbour table [(q-1)][nf]
     int64_t launches = 0;
-    unsigned int* dtimeouts = nullptr;  // device counter of staged-copy waits that ran out
+    unsigned int* dtimeouts = nullptr;  // device counter of bounded waits that ran out
+    bool selftest = false;      // a self-test was queued since it was read: no step waits
     bool compact = false;       // compact layout: dense records, work split by tile column
     double cthr = 0.3;          // compact: fluid fraction from which a tile column is tiled
     bool c_tiled_ok = false;    // compact: the box is whole tile columns, and the tiled kernel takes those dense enough
@@ -114,12 +115,13 @@ void free_all(lbm_tau1* h)
     if (h->cnodes) cudaFree(h->cnodes);
 }
 
-// Staged-copy waits that ran out since the last call (reads the device
+// Bounded waits that ran out since the last call (reads the device
 // counter on the handle's stream, then clears it).
 unsigned int take_timeouts(lbm_tau1* h)
 {
     unsigned int v = 0;
-    if (!h->dtimeouts) return 0;
+    if (!h->dtimeouts || !h->selftest) return 0;
+    h->selftest = false;
     if (cudaMemcpyAsync(&v, h->dtimeouts, sizeof(v), cudaMemcpyDefault, h->stream) != cudaSuccess) return 0;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return 0;
     if (v) cudaMemsetAsync(h->dtimeouts, 0, sizeof(v), h->stream);
@@ -151,7 +153,6 @@ void fill_args(const lbm_tau1* h, StepArgs& a)
     a.post = h->buf[h->cur ^ 1];
     a.dscale = h->dscale;
     a.seed = (uint32_t)(h->step + 1) * 0x9E3779B9u;
-    a.timeouts = h->dtimeouts;
     for (int f = 0; f < 4; ++f) {
         a.inv_scale[f] = h->inv_scale[f];
         a.scale[f] = h->scale[f];
@@ -632,7 +633,7 @@ lbm_status lbm_tau1_synchronize(lbm_tau1* h)
     if (!h) return fail(nullptr, LBM_EINVAL, "synchronize: NULL handle");
     LBM_CUDA(h, cudaStreamSynchronize(h->stream), "synchronize");
     if (unsigned t = take_timeouts(h))
-        return fail(h, LBM_ETIMEOUT, "synchronize: " + std::to_string(t) + " staged-copy waits ran out");
+        return fail(h, LBM_ETIMEOUT, "synchronize: " + std::to_string(t) + " bounded waits ran out");
     return LBM_OK;
 }
 
@@ -854,6 +855,7 @@ lbm_status lbm_tau1_selftest_timeout(lbm_tau1* h)
 {
     if (!h) return fail(nullptr, LBM_EINVAL, "selftest_timeout: NULL handle");
     LBM_CUDA(h, launch_selftest_timeout(h->dtimeouts, h->stream), "selftest_timeout: launch");
+    h->selftest = true;
     ++h->launches;
     return LBM_OK;
 }
@@ -976,7 +978,7 @@ lbm_status lbm_tau1_reduce(lbm_tau1* h, lbm_tau1_stats* out)
                                 h->stream), "reduce: copy");
     LBM_CUDA(h, cudaStreamSynchronize(h->stream), "reduce: sync");
     if (unsigned t = take_timeouts(h))
-        return fail(h, LBM_ETIMEOUT, "reduce: " + std::to_string(t) + " staged-copy waits ran out");
+        return fail(h, LBM_ETIMEOUT, "reduce: " + std::to_string(t) + " bounded waits ran out");
     const lbm_status st = fill_stats(h->red_host, h->n, h->cfg.g, h->step, out);
     h->n_fluid = out->n_fluid;
     if (st == LBM_EDIVERGED) return fail(h, st, "reduce: state diverged (non-finite value or |u| > 0.3)");

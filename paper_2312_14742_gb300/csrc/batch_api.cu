@@ -64,7 +64,9 @@ struct lbm_tau1_batch {
     double* red_partials = nullptr;
     double* red_out = nullptr;   // device [capacity][RED_FIELDS]
     double* red_host = nullptr;  // pinned copy
-    unsigned int* dtimeouts = nullptr;  // device counter of staged-copy waits that ran out
+    unsigned int* dtimeouts = nullptr;  // device counter of bounded waits that ran out
+    bool selftest = false;   // a self-test was queued since it was read: no step waits
+    bool qselftest = false;  // the queued statistics carry its count
     // queued statistics (stats_queue / stats_wait): their own device and
     // pinned buffers ([capacity][RED_FIELDS], then the timeout count), the
     // event after the copy, and what the host needs to finish them
@@ -88,12 +90,13 @@ lbm_status bfail(lbm_tau1_batch* b, lbm_status st, const std::string& msg)
     return st;
 }
 
-// Staged-copy waits that ran out since the last call (the caller has
+// Bounded waits that ran out since the last call (the caller has
 // synchronised the batch's stream); clears the counter.
 unsigned int take_timeouts(lbm_tau1_batch* b)
 {
     unsigned int v = 0;
-    if (!b->dtimeouts) return 0;
+    if (!b->dtimeouts || !b->selftest) return 0;
+    b->selftest = false;
     if (cudaMemcpy(&v, b->dtimeouts, sizeof(v), cudaMemcpyDefault) != cudaSuccess) return 0;
     if (v) cudaMemset(b->dtimeouts, 0, sizeof(v));
     return v;
@@ -409,7 +412,6 @@ lbm_status lbm_tau1_batch_admit(lbm_tau1_batch* b, const lbm_tau1_config* cfg, c
     rec.a.nx = cfg->nx;
     rec.a.ny = cfg->ny;
     rec.a.nz = cfg->nz;
-    rec.a.timeouts = b->dtimeouts;
     for (int d = 0; d < 3; ++d) {
         rec.a.periodic[d] = per[d];
         rec.a.g[d] = cfg->g[d];
@@ -507,7 +509,7 @@ lbm_status lbm_tau1_batch_stats(lbm_tau1_batch* b, int32_t n, const int32_t* slo
                              b->stream), "batch_stats: copy");
     BCUDA(b, cudaStreamSynchronize(b->stream), "batch_stats: sync");
     if (unsigned t = take_timeouts(b))
-        return bfail(b, LBM_ETIMEOUT, "batch_stats: " + std::to_string(t) + " staged-copy waits ran out");
+        return bfail(b, LBM_ETIMEOUT, "batch_stats: " + std::to_string(t) + " bounded waits ran out");
     lbm_status worst = LBM_OK;
     for (int i = 0; i < n; ++i) {
         const Slot& s = b->slots[slots[i]];
@@ -522,6 +524,7 @@ lbm_status lbm_tau1_batch_selftest_timeout(lbm_tau1_batch* b)
 {
     if (!b) return bfail(nullptr, LBM_EINVAL, "batch_selftest_timeout: NULL batch");
     BCUDA(b, launch_selftest_timeout(b->dtimeouts, b->stream), "batch_selftest_timeout: launch");
+    b->selftest = true;
     ++b->launches;
     return LBM_OK;
 }
@@ -547,14 +550,18 @@ lbm_status lbm_tau1_batch_stats_queue(lbm_tau1_batch* b, int32_t n, const int32_
         b->qsteps[(size_t)i] = s.steps;
         b->qcfg[(size_t)i] = s.cfg;
     }
-    // the statistics and the timeout count (as a double after them), then the count cleared
+    // the statistics; after a self-test the timeout count behind them, then the count cleared
     const size_t tail = (size_t)n * RED_FIELDS;
     BCUDA(b, cudaMemcpyAsync(b->qred_host, b->qred_out, tail * sizeof(double), cudaMemcpyDefault, b->stream),
           "batch_stats_queue: copy");
-    unsigned int* tcount = reinterpret_cast<unsigned int*>(b->qred_host + tail);
-    BCUDA(b, cudaMemcpyAsync(tcount, b->dtimeouts, sizeof(unsigned int), cudaMemcpyDefault, b->stream),
-          "batch_stats_queue: copy");
-    BCUDA(b, cudaMemsetAsync(b->dtimeouts, 0, sizeof(unsigned int), b->stream), "batch_stats_queue: clear");
+    b->qselftest = b->selftest;
+    if (b->selftest) {
+        unsigned int* tcount = reinterpret_cast<unsigned int*>(b->qred_host + tail);
+        BCUDA(b, cudaMemcpyAsync(tcount, b->dtimeouts, sizeof(unsigned int), cudaMemcpyDefault, b->stream),
+              "batch_stats_queue: copy");
+        BCUDA(b, cudaMemsetAsync(b->dtimeouts, 0, sizeof(unsigned int), b->stream), "batch_stats_queue: clear");
+        b->selftest = false;
+    }
     BCUDA(b, cudaEventRecord(b->qev, b->stream), "batch_stats_queue: event");
     b->qpending = true;
     return LBM_OK;
@@ -568,8 +575,8 @@ lbm_status lbm_tau1_batch_stats_wait(lbm_tau1_batch* b, lbm_tau1_stats* out)
     if (n > 0 && !out) return bfail(b, LBM_EINVAL, "batch_stats_wait: NULL output");
     b->qpending = false;
     BCUDA(b, cudaEventSynchronize(b->qev), "batch_stats_wait: sync");
-    const unsigned int t = *reinterpret_cast<const unsigned int*>(b->qred_host + (size_t)n * RED_FIELDS);
-    if (t) return bfail(b, LBM_ETIMEOUT, "batch_stats_wait: " + std::to_string(t) + " staged-copy waits ran out");
+    const unsigned int t = b->qselftest ? *reinterpret_cast<const unsigned int*>(b->qred_host + (size_t)n * RED_FIELDS) : 0;
+    if (t) return bfail(b, LBM_ETIMEOUT, "batch_stats_wait: " + std::to_string(t) + " bounded waits ran out");
     lbm_status worst = LBM_OK;
     for (int i = 0; i < n; ++i)
         if (fill_stats(b->qred_host + (size_t)i * RED_FIELDS, b->qn[(size_t)i], b->qcfg[(size_t)i].g,
@@ -611,7 +618,7 @@ lbm_status lbm_tau1_batch_synchronize(lbm_tau1_batch* b)
     if (!b) return bfail(nullptr, LBM_EINVAL, "batch_synchronize: NULL batch");
     BCUDA(b, cudaStreamSynchronize(b->stream), "batch_synchronize");
     if (unsigned t = take_timeouts(b))
-        return bfail(b, LBM_ETIMEOUT, "batch_synchronize: " + std::to_string(t) + " staged-copy waits ran out");
+        return bfail(b, LBM_ETIMEOUT, "batch_synchronize: " + std::to_string(t) + " bounded waits ran out");
     return LBM_OK;
 }
 

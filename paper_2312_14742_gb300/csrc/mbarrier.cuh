@@ -1,9 +1,9 @@
 // Shared-memory addresses and bounded mbarrier waits.
 //
 // A wait that runs past its limit returns false; its kernel then counts a
-// timeout in its caller's device counter (StepArgs::timeouts, read and cleared
-// by the host, which reports LBM_ETIMEOUT) and returns, so that a missing
-// completion can never hang the GPU.
+// timeout in a device counter (read and cleared by the host, which reports
+// LBM_ETIMEOUT) and returns, so that a missing completion can never hang the GPU.
+// No step kernel waits; the self-test (selftest.cu) does.
 #pragma once
 
 #include <cstdint>
@@ -20,11 +20,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
 
 // makes initialised barriers visible to the asynchronous (TMA) proxy
 __device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
 {

@@ -1,7 +1,7 @@
-// Self-test of the failure detection of the staged kernels: a wait on an
-// mbarrier whose phase nothing completes, with the same bounded wait and the
-// same device counter as the step kernels, so that a test or a health check
-// can see a wait run out and reach the host as LBM_ETIMEOUT without any fault.
+// Self-test of the failure detection: a wait on an mbarrier whose phase nothing
+// completes, bounded, and counted in the handle's device counter, so that a test
+// or a health check can see a wait run out and reach the host as LBM_ETIMEOUT
+// without any fault.
 #include "kernels.h"
 #include "mbarrier.cuh"
 
