@@ -7,13 +7,13 @@
 // depend on the chunk. A grid of (SMs x resident blocks) works through the list:
 // each warp takes its first item by its index and then the next unclaimed one
 // (an atomic counter), so warps that drew small items (partial strips or chunks)
-// take more of them. Each item is one strip_step() call with that box's
-// arguments, read from the device table. Everything that changes from step to
+// take more of them. Each item is one strip_step() or strip_links() call with that
+// box's arguments, read from the device table. Everything that changes from step to
 // step lives in the table on the device: which copy holds a box's current
 // state, its step count (the stochastic-rounding seed), its 16-bit scales.
-// Boxes of every size take the same strips (strip.cuh). A launch therefore has the same arguments every step, and K steps can be
-// captured once in a CUDA graph and replayed while boxes come and go (the host
-// edits the table between replays).
+// Boxes of every size take the same strips (strip.cuh). A launch therefore has the
+// same arguments every step, and K steps can be captured once in a CUDA graph and
+// replayed while boxes come and go (the host edits the table between replays).
 //
 // The last block to finish (an atomic count, no waiting) closes the step for
 // every live box: swaps its copies, counts the step and, for FP16 storage,
@@ -181,10 +181,18 @@ struct BatchKernel {
     }
 };
 
-// Shape of variant 0; the others name one. The arguments that come from the table
-// take registers: the formats summed link by link take the shape that spills
-// nothing, or next to nothing.
-constexpr int batch_shape(int q, int st) { return st == ST_BF16S ? 0 : 1; }
+// Shape of variant 0; the others name one. The arguments come from the table and
+// take registers, so that the formats summed link by link do not all take the shape
+// of the single box. us per step of 12 boxes of 32^3 to 128^3, of 4 of 192^3 and of
+// 3 of 96^3, with shape 0, 1 and 2: D3Q19 FP16 101, 117, 96; 273, 271, 274; 37, 40, 36;
+// BF16 94, 108, 92; 256, 256, 263; 34, 38, 34; D3Q27 FP16 162, 145, 157; 377, 377, 419;
+// 54, 49, 52; BF16 144, 138, 132; 347, 364, 364; 50, 47, 46.
+constexpr int batch_shape(int q, int st)
+{
+    if (st == ST_F16S) return q == 19 ? 2 : 1;
+    if (st == ST_BF16S) return q == 19 ? 0 : 2;
+    return 1;
+}
 
 template <int Q, int ST>
 cudaError_t dispatch_v(int variant, bool prep, BatchTable* T, int& grid, int& rows, cudaStream_t s)
