@@ -173,8 +173,8 @@ def paper_baseline(args):
             "source": "Table tab:perf_comp, D2Q9 on 4000^2"}
 
 
-TILED_KERNEL_SOURCES = ("tau1_strip.cu", "strip.cuh", "moments.cuh", "links.cuh", "tau1_node.cuh", "mbarrier.cuh", "pack2.cuh", "common.cuh",
-                        "lattice.cuh", "static_for.cuh", "kernels.h")
+TILED_KERNEL_SOURCES = ("tau1_strip.cu", "strip.cuh", "strip_plan.h", "moments.cuh", "links.cuh", "tau1_node.cuh",
+                        "mbarrier.cuh", "pack2.cuh", "common.cuh", "lattice.cuh", "static_for.cuh", "kernels.h")
 
 
 def kernel_source_hash() -> str:

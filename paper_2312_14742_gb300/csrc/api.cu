@@ -308,9 +308,9 @@ lbm_status build_fluid_list(lbm_tau1* h)
     return LBM_OK;
 }
 
-// Compact layout: classes the tile columns of variant h->variant by their fluid counts (counted once per geometry and variant)
-// with threshold h->cthr and uploads the two lists; the node list is written
-// by a kernel from the flags.
+// Compact layout: classes the tile columns of variant h->variant by their fluid
+// counts (counted once per geometry and variant) with threshold h->cthr and uploads
+// the two lists; the node list is written by a kernel from the flags.
 lbm_status build_compact(lbm_tau1* h)
 {
     const lbm_tau1_config& c = h->cfg;

@@ -147,8 +147,8 @@ cudaError_t stage_done(Stage* s, cudaStream_t stream)
 int64_t box_items(const Slot& s, int chunk) { return (int64_t)s.nstrips * (((int64_t)s.cfg.nz + chunk - 1) / chunk); }
 
 // Rebuilds the live list and item offsets and queues their upload. The chunk
-// is the one with the least (waves of items over the persistent grid's warps) x (planes
-// an item forms: two beside its own, and about as much again to start).
+// is the one with the least (waves of items over the persistent grid's warps) x
+// (planes an item forms: two beside its own, and about as much again to start).
 lbm_status upload_table(lbm_tau1_batch* b)
 {
     static const int chunks[] = {64, 48, 40, 32, 28, 24, 20, 16, 12, 10, 8, 6, 5, 4, 3, 2};

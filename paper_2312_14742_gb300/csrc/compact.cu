@@ -64,14 +64,19 @@ __device__ __forceinline__ void axis_sources(uint32_t c, uint32_t n, int st, boo
 // gathered from the dense state. A source outside a non-periodic face is read
 // from the sentinel record n (drho = NaN, u = 0) that follows the box in both
 // state copies, so that every source is a plain load and a wall is recognised by
-// its NaN alone. The sums are those of moments.cuh or links.cuh. One thread per node: two
-// nodes per thread in packed arithmetic take a third fewer instructions but
-// leave too few warps to hide the gathers (303 us against 256 on 9.9 M nodes).
+// its NaN alone. The sums are those of moments.cuh or links.cuh. One thread per
+// node: two nodes per thread in packed arithmetic take a third fewer instructions
+// but leave too few warps to hide the gathers (303 us against 256 on 9.9 M nodes).
+// Warps matter more than loads in flight per thread: at 40 registers (D3Q19) a
+// thread cannot hold 18 records, and the compiler spreads the loads that are
+// written first; D3Q27 with all 26 records in registers takes 341 to 416 us.
 // Away from the faces, where all nodes of a warp are as a rule, the sources lie at
-// fixed distances: a third of the instructions went into finding them. 9.9 M
-// nodes in D3Q19 take 204 us (221 without that case, 238 link by link), in D3Q27
-// 345 (359, 342); the default split of the same box (320^3, 30% fluid) 199 us
-// and 258, where the link-by-link kernels took 225 and 351.
+// fixed distances: a third of the instructions went into finding them. 9.9 M nodes
+// in D3Q19 take 204 us (221 without that case, 236 link by link), in D3Q27 321 (336,
+// 339), in BF16 222 and 311 (244 and 331 before the strips); the default split of the
+// same box (320^3, 30% fluid) 203 us and 258, 211 and 350 before the strips. D3Q27
+// boxes that stay in L2 and go to the list altogether are slower than link by link:
+// 161 x 127 x 101 at 40% 30.8 us against 28.8.
 struct ListArgs {
     const int* nodes;
     int count;
@@ -120,7 +125,7 @@ __global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12
     if (isnan(r[0].d)) return;  // a listed node is fluid; a NaN state is left as it is, as elsewhere
     auto step = [&](auto source) {
         constexpr bool FIRST = sizeof(T) == 4 && (Q == 19 || by_links(ST));
-        if constexpr (FIRST)  // every load first (else as they are used, for registers)
+        if constexpr (FIRST)  // loads first (else as they are used)
             static_for<1, Q>([&](auto kc) { load(r[decltype(kc)::value], source(kc)); });
         auto fetch = [&](auto kc, bool& solid) -> const Rec<T>& {
             constexpr int K = decltype(kc)::value;

@@ -129,12 +129,12 @@ __global__ void __launch_bounds__(256) table_kernel(int nf, int nx, int ny, int 
 }
 
 // One Tau1 step of the fluid list: one thread per fluid node. D3Q19 hides the
-// latency of its gathers with warps (32 registers: 52.5 us for 1.8 M nodes, 61
-// with the registers the compiler would take); D3Q27 does better with more loads
-// in flight per thread (72 us against 95 at 40 registers). Summing link by link
-// took 55.5 and 82 us in FP32. The 16-bit formats do (links.cuh): BF16 51 and 70 us
-// with the indices first (59 and 93 each as it is used), FP16 54 and 81, where a
-// wall skips the scaling of a record (60 and 84 with the bounds of BF16).
+// latency of its gathers with warps (32 registers and 56 bytes of spills: 52.5 us
+// for 1.8 M nodes, 61 with the registers the compiler would take); D3Q27 does better
+// with more loads in flight per thread (72 us against 95 at 40 registers). Summing
+// link by link took 55.5 and 82 us in FP32. The 16-bit formats do (links.cuh): BF16
+// 52 and 70 us with the indices first (59 and 93 each as it is used), FP16 52 and 80,
+// where a wall skips the scaling of a record (60 and 84 with the bounds of BF16).
 constexpr int sparse_blocks(int q, int st)
 {
     return st == ST_F32 && q == 19 ? 8 : (st == ST_BF16S ? (q == 19 ? 6 : 4) : 0);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256, sparse_blocks(Q, ST)) tau1_sparse_kernel(
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf) return;
     const Scales sc(a.dscale);
-    // every index first: the records' loads then wait for none but their own
+    // the indices first, so that few loads of records wait for one
     int src[Q];
     static_for<1, Q>([&](auto kc) {
         constexpr int K = decltype(kc)::value;

@@ -26,12 +26,12 @@
 // The 16-bit formats march the same strips link by link (strip_links()): no list,
 // and more values along x.
 //
-// 256^3, spheres of radius 8 at 90% porosity: D3Q19 FP32 137 us per step (the
-// link-by-link row-pair kernel before it 155), BF16 150 (183), D3Q27 FP32 146
-// (247), BF16 206 (315); 128^3 D3Q19 FP64 660 (937). FP32 is bound by issue and the latency
-// of its 12 warps per SM, not by HBM (74 us for the state alone). Blocks whose
-// four warps met at a barrier per plane and formed 32 own columns each took 149,
-// 173, 175 and 729.
+// 256^3, spheres of radius 8 at 90% porosity, us per step by default, and of the
+// tile kernels before: D3Q19 FP32 136 (156), BF16 150 (183), D3Q27 FP32 147 (261), BF16
+// 206 (315); 128^3 D3Q19 FP64 702 (934). FP32 is bound by issue and the latency of
+// the 12 warps per SM of four-row strips, not by HBM (74 us for the state alone).
+// Blocks whose four warps met at a barrier per plane and formed 32 own columns each
+// took 10 to 23% more.
 #pragma once
 
 #include "kernels.h"
