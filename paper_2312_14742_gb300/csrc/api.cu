@@ -58,6 +58,8 @@ struct lbm_tau1 {
     std::vector<int> ccounts_host;
     int* cstrips = nullptr;     // compact: strips of the tiled kernel [cscap], n_cstrips of them
     int64_t cscap = 0, n_cstrips = 0;
+    int czstrip = 0;            // compact: planes per strip
+    bool cstrips_first = false; // compact: the strips are launched before the node list
     int* clisted = nullptr;     // compact: tile columns of the node list, then their offsets [2 columns]
     int* cnodes = nullptr;      // compact: the node list [fluid nodes]
     int64_t n_ctiles = 0, n_clisted = 0, n_cnodes = 0, c_tiled_fluid = 0, c_empty = 0;
@@ -364,7 +366,12 @@ lbm_status build_compact(lbm_tau1* h)
     h->n_clisted = (int64_t)offsets.size();
     h->n_cnodes = nodes;
     std::vector<int> items;
-    compact_strips(ct, c.nx, c.ny, c.nz, tiles, items);
+    compact_strips(ct, c.nx, c.ny, c.nz, tiles, ct.zchunk, items);
+    const CompactPlan plan = compact_plan(c.q, c.storage, ct.shape, ct.zchunk, (int64_t)(items.size() / STRIP_ITEM),
+                                          nodes, h->sms);
+    h->czstrip = plan.planes;
+    h->cstrips_first = plan.first;
+    if (h->czstrip != ct.zchunk) compact_strips(ct, c.nx, c.ny, c.nz, tiles, h->czstrip, items);
     h->n_cstrips = (int64_t)(items.size() / STRIP_ITEM);
     if ((int64_t)items.size() > h->cscap) {
         if (h->cstrips) { cudaFree(h->cstrips); h->cstrips = nullptr; }
@@ -406,15 +413,20 @@ cudaError_t launch_kernel(const lbm_tau1* h, const StripPlan& plan, const StepAr
 {
     if (h->cfg.q == LBM_D2Q9) return launch_tau1_2d(h->kernel == LBM_KERNEL_SIMPLE, h->cfg.storage, a, h->stream);
     if (h->compact) {
-        // Disjoint node sets, both read from the same copy: the tiled kernel may
-        // start as soon as the last blocks of the node-list kernel have (it fills
-        // the SMs that their tail leaves idle). With the list on a stream of its
-        // own it was a race which of the two got the SMs first: 211 us per step
-        // (320^3, 30% fluid) where the list did, 249 us where the tiled blocks did.
-        cudaError_t e = launch_tau1_list(h->cfg.q, h->cfg.storage, a, h->cnodes, h->n_cnodes, h->stream);
-        if (e == cudaSuccess)
-            e = launch_tau1_tiled_list(h->cfg.q, h->cfg.storage, h->ctile.shape, h->ctile.zchunk, a, h->cstrips,
-                                       (int)h->n_cstrips, h->n_cnodes > 0, h->stream);
+        // Disjoint node sets, both read from the same copy: the second kernel may
+        // start as soon as the last blocks of the first have. With the list on a
+        // stream of its own it was a race which of the two got the SMs first: 211 us
+        // per step (320^3, 30% fluid) where the list did, 249 us where tiles did.
+        const bool both = h->n_cnodes > 0 && h->n_cstrips > 0;
+        auto strips = [&](bool second) {
+            return launch_tau1_tiled_list(h->cfg.q, h->cfg.storage, h->ctile.shape, h->czstrip, a, h->cstrips,
+                                          (int)h->n_cstrips, second ? h->sms : 0, h->stream);
+        };
+        auto nodes = [&](bool second) {
+            return launch_tau1_list(h->cfg.q, h->cfg.storage, a, h->cnodes, h->n_cnodes, second, h->stream);
+        };
+        cudaError_t e = h->cstrips_first ? strips(false) : nodes(false);
+        if (e == cudaSuccess) e = h->cstrips_first ? nodes(both) : strips(both);
         return e;
     }
     if (h->sparse) return launch_tau1_sparse(h->cfg.q, h->cfg.storage, a, (int)h->nf, h->nbr, h->stream);

@@ -74,7 +74,7 @@ __device__ __forceinline__ void axis_sources(uint32_t c, uint32_t n, int st, boo
 // fixed distances: a third of the instructions went into finding them. 9.9 M nodes
 // in D3Q19 take 204 us (221 without that case, 236 link by link), in D3Q27 321 (336,
 // 339), in BF16 222 and 311 (244 and 331 before the strips); the default split of the
-// same box (320^3, 30% fluid) 203 us and 258, 211 and 350 before the strips. D3Q27
+// same box (320^3, 30% fluid) 205 us and 249, 211 and 350 before the strips. D3Q27
 // boxes that stay in L2 and go to the list altogether are slower than link by link:
 // 161 x 127 x 101 at 40% 30.8 us against 28.8.
 struct ListArgs {
@@ -108,11 +108,10 @@ struct Around {
     }
 };
 
-template <int Q, int ST>
-__global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12 : 8)) tau1_list_kernel(StepArgs a, ListArgs l)
+// The step of the listed node of this thread.
+template <int Q, int ST> __device__ __forceinline__ void list_node(const StepArgs& a, const ListArgs& l)
 {
     using T = typename Storage<ST>::ctype;
-    asm volatile("griddepcontrol.launch_dependents;");  // the tiled kernel of this step: other nodes
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const Scales sc(a.dscale);
     const uint32_t sentinel = (uint32_t)a.nx * (uint32_t)a.ny * (uint32_t)a.nz;
@@ -170,6 +169,15 @@ __global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12
     }
 }
 
+template <int Q, int ST>
+__global__ void __launch_bounds__(LIST_THREADS, ST == ST_F64 ? 0 : (Q == 19 ? 12 : 8)) tau1_list_kernel(StepArgs a, ListArgs l)
+{
+    asm volatile("griddepcontrol.launch_dependents;");  // the tiled kernel of this step: other nodes
+    list_node<Q, ST>(a, l);
+    // a launch that began before the tiled kernel had ended ends after it
+    if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The sentinel record n of a state copy: drho = NaN, u = 0.
 template <int ST>
 __global__ void sentinel_kernel(void* buf, uint32_t n, const float* __restrict__ dscale)
@@ -180,11 +188,19 @@ __global__ void sentinel_kernel(void* buf, uint32_t n, const float* __restrict__
 }
 
 template <int Q, int ST>
-cudaError_t launch_list_t(const StepArgs& a, const int* nodes, int count, cudaStream_t s)
+cudaError_t launch_list_t(const StepArgs& a, const int* nodes, int count, bool after_tiled, cudaStream_t s)
 {
     const ListArgs l{nodes, count, DivBy::make((uint32_t)a.nx), DivBy::make((uint32_t)a.nx * (uint32_t)a.ny)};
-    tau1_list_kernel<Q, ST><<<(unsigned)((count + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0, s>>>(a, l);
-    return cudaGetLastError();
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((count + LIST_THREADS - 1) / LIST_THREADS));
+    cfg.blockDim = dim3(LIST_THREADS);
+    cfg.stream = s;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = after_tiled ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, tau1_list_kernel<Q, ST>, a, l);
 }
 
 constexpr int CT = 256;  // threads of the count and list kernels (8 warps)
@@ -285,8 +301,10 @@ CompactTiles compact_tiles(int q, int storage, int variant)
     const int nr = tau1_tile_shapes(storage);
     CompactTiles t;
     const int v = variant % nr;
-    // four rows per strip, two for v 2, 3; link by link two, and another register budget for v 2, 3
-    t.shape = nr == 1 ? 0 : ((v < 2) != by_links(storage) ? 1 : 0);
+    // two rows per strip, for v 2, 3 four (link by link another register budget): a list
+    // of few strips is balanced by halves (D3Q19 FP32 at 30% fluid: 192^3 61.6 and 59.6 us
+    // with four rows and two, 256^3 122.6 and 118.7, 320^3 206.0 and 204.7)
+    t.shape = nr == 1 || v < 2 ? 0 : 1;
     t.zchunk = variant < nr ? 24 : 32;
     t.h = v == 1 ? 16 : (v == 3 ? 12 : 8);
     t.rows = strip_shape(q, storage, t.shape).rows;
@@ -312,7 +330,8 @@ int64_t compact_tile_nodes(const CompactTiles& t, int nx, int ny, int nz, int b)
     return w * hh * d;
 }
 
-void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, std::vector<int>& items)
+void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, int zstrip,
+                    std::vector<int>& items)
 {
     const TileGeo g = geo_of(t, nx, ny, nz);
     items.clear();
@@ -321,30 +340,37 @@ void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::ve
         for (; lanes < 32; ++lanes) items.push_back(items.back() < 0 ? items.back() : ~items.back());
         if (chunk >= 0) items.push_back(chunk);
     };
-    for (size_t i = 0; i < tiles.size();) {
-        // a run of tiles side by side, then each of its groups of rows
-        const int tile = tiles[i] % g.ntiles, c = tiles[i] / g.ntiles, tx = tile % g.ntx;
-        size_t e = i + 1;
-        while (e < tiles.size() && tiles[e] == tiles[e - 1] + 1 && tx + (int)(e - i) < g.ntx) ++e;
-        for (int j = 0; j < t.h / t.rows; ++j) {
-            const int first = (tile / g.ntx * (t.h / t.rows) + j) * (nx + 2);  // slot of column -1
-            int x = 32 * tx;
-            const int end = std::min(nx, 32 * (tx + (int)(e - i)));
-            while (x < end) {
-                if (lanes > 29 || c != chunk) {
-                    pad();
-                    lanes = 0;
-                    chunk = c;
+    for (size_t first = 0, last; first < tiles.size(); first = last) {
+        // the tiles of one chunk of planes, once for each of its parts
+        const int c = tiles[first] / g.ntiles, z1 = std::min(nz, (c + 1) * g.chunk);
+        for (last = first; last < tiles.size() && tiles[last] / g.ntiles == c;) ++last;
+        for (int z0 = c * g.chunk; z0 < z1; z0 += zstrip) {
+            for (size_t i = first; i < last;) {
+                // a run of tiles side by side, then each of its groups of rows
+                const int tile = tiles[i] % g.ntiles, tx = tile % g.ntx;
+                size_t e = i + 1;
+                while (e < last && tiles[e] == tiles[e - 1] + 1 && tx + (int)(e - i) < g.ntx) ++e;
+                for (int j = 0; j < t.h / t.rows; ++j) {
+                    const int row = (tile / g.ntx * (t.h / t.rows) + j) * (nx + 2);  // slot of column -1
+                    int x = 32 * tx;
+                    const int end = std::min(nx, 32 * (tx + (int)(e - i)));
+                    while (x < end) {
+                        if (lanes > 29 || z0 / zstrip != chunk) {
+                            pad();
+                            lanes = 0;
+                            chunk = z0 / zstrip;
+                        }
+                        const int n = std::min(end - x, 30 - lanes);
+                        items.push_back(~(row + x));
+                        for (int k = 1; k <= n; ++k) items.push_back(row + x + k);
+                        items.push_back(~(row + x + n + 1));
+                        lanes += n + 2;
+                        x += n;
+                    }
                 }
-                const int n = std::min(end - x, 30 - lanes);
-                items.push_back(~(first + x));
-                for (int k = 1; k <= n; ++k) items.push_back(first + x + k);
-                items.push_back(~(first + x + n + 1));
-                lanes += n + 2;
-                x += n;
+                i = e;
             }
         }
-        i = e;
     }
     pad();
 }
@@ -380,21 +406,22 @@ cudaError_t launch_compact_sentinel(int storage, void* buf, int64_t n, const flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_tau1_list(int q, int storage, const StepArgs& a, const int* nodes, int64_t count, cudaStream_t s)
+cudaError_t launch_tau1_list(int q, int storage, const StepArgs& a, const int* nodes, int64_t count, bool after_tiled,
+                             cudaStream_t s)
 {
     if (count == 0) return cudaSuccess;
     // node indices are int32 and nx ny z + y nx + x must not wrap in 32 bits
     if (count > 0x7fffffffLL || (int64_t)a.nx * a.ny * a.nz >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
     const int c = (int)count;
     switch (q * 10 + storage) {
-    case 190 + ST_F64: return launch_list_t<19, ST_F64>(a, nodes, c, s);
-    case 190 + ST_F32: return launch_list_t<19, ST_F32>(a, nodes, c, s);
-    case 190 + ST_F16S: return launch_list_t<19, ST_F16S>(a, nodes, c, s);
-    case 190 + ST_BF16S: return launch_list_t<19, ST_BF16S>(a, nodes, c, s);
-    case 270 + ST_F64: return launch_list_t<27, ST_F64>(a, nodes, c, s);
-    case 270 + ST_F32: return launch_list_t<27, ST_F32>(a, nodes, c, s);
-    case 270 + ST_F16S: return launch_list_t<27, ST_F16S>(a, nodes, c, s);
-    case 270 + ST_BF16S: return launch_list_t<27, ST_BF16S>(a, nodes, c, s);
+    case 190 + ST_F64: return launch_list_t<19, ST_F64>(a, nodes, c, after_tiled, s);
+    case 190 + ST_F32: return launch_list_t<19, ST_F32>(a, nodes, c, after_tiled, s);
+    case 190 + ST_F16S: return launch_list_t<19, ST_F16S>(a, nodes, c, after_tiled, s);
+    case 190 + ST_BF16S: return launch_list_t<19, ST_BF16S>(a, nodes, c, after_tiled, s);
+    case 270 + ST_F64: return launch_list_t<27, ST_F64>(a, nodes, c, after_tiled, s);
+    case 270 + ST_F32: return launch_list_t<27, ST_F32>(a, nodes, c, after_tiled, s);
+    case 270 + ST_F16S: return launch_list_t<27, ST_F16S>(a, nodes, c, after_tiled, s);
+    case 270 + ST_BF16S: return launch_list_t<27, ST_BF16S>(a, nodes, c, after_tiled, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -23,10 +23,11 @@ int tau1_tile_shapes(int storage);
 // strip STRIP_ITEM ints, its 32 slots (ys (nx + 2) + x + 1 for column x of the
 // ys-th group of rows; ~slot where the strip does not own the column) and its
 // chunk of zchunk planes. An owned column has its neighbours in the next lanes.
-// after_list: the last launch on s is launch_tau1_list() of the same step.
+// after_list: 0, or the SMs of the device if the last launch on s is
+// launch_tau1_list() of the same step, beside whose last blocks these may start.
 constexpr int STRIP_ITEM = 33;
 cudaError_t launch_tau1_tiled_list(int q, int storage, int shape, int zchunk, const StepArgs& a, const int* list,
-                                   int count, bool after_list, cudaStream_t s);
+                                   int count, int after_list, cudaStream_t s);
 // Self-test (selftest.cu): one warp waits, bounded, on an mbarrier phase
 // that nothing completes and counts the timeout in *timeouts.
 cudaError_t launch_selftest_timeout(unsigned int* timeouts, cudaStream_t s);
@@ -42,10 +43,11 @@ struct CompactTiles {
 CompactTiles compact_tiles(int q, int storage, int variant);
 int64_t compact_tile_columns(const CompactTiles& t, int nx, int ny, int nz);
 int64_t compact_tile_nodes(const CompactTiles& t, int nx, int ny, int nz, int b);
-// The strips that cover the given tile columns (in grid order), as
-// launch_tau1_tiled_list takes them; the box is whole tiles (nx a multiple of 32,
-// ny of the tile height).
-void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, std::vector<int>& items);
+// The strips of zstrip planes (a divisor of t.zchunk) that cover the given tile
+// columns (in grid order), as launch_tau1_tiled_list takes them; the box is whole
+// tiles (nx a multiple of 32, ny of the tile height).
+void compact_strips(const CompactTiles& t, int nx, int ny, int nz, const std::vector<int>& tiles, int zstrip,
+                    std::vector<int>& items);
 cudaError_t launch_compact_count(const CompactTiles& t, int nx, int ny, int nz, const uint8_t* flags, int* counts,
                                  cudaStream_t s);
 cudaError_t launch_compact_nodes(const CompactTiles& t, int nx, int ny, int nz, const uint8_t* flags, const int* tiles,
@@ -53,9 +55,11 @@ cudaError_t launch_compact_nodes(const CompactTiles& t, int nx, int ny, int nz, 
 // Tau1 step of the listed box nodes (fluid), one thread per node, the
 // neighbours gathered from the dense records (the dense kernels' values); the
 // state copies hold n + 1 records, record n the solid sentinel written by
-// launch_compact_sentinel (dscale: the 16-bit scales, or NULL).
+// launch_compact_sentinel (dscale: the 16-bit scales, or NULL). after_tiled: the last
+// launch on s is launch_tau1_tiled_list() of the same step, beside which it may start.
 cudaError_t launch_compact_sentinel(int storage, void* buf, int64_t n, const float* dscale, cudaStream_t s);
-cudaError_t launch_tau1_list(int q, int storage, const StepArgs& a, const int* nodes, int64_t count, cudaStream_t s);
+cudaError_t launch_tau1_list(int q, int storage, const StepArgs& a, const int* nodes, int64_t count, bool after_tiled,
+                             cudaStream_t s);
 
 // D2Q9 (one plane): simple = one thread per node, else the y-marching warp
 // kernel; same bits.

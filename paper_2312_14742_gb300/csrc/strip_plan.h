@@ -52,14 +52,14 @@ constexpr StripShapeCost strip_shape(int q, int storage, int v)
                   : (v == 1 ? StripShapeCost{2, 2, {0, 0.87, 1.2, 0, 0}} : StripShapeCost{4, 2, {0, 1.6, 2.3, 0, 0}});
 }
 
-// Time of a step of nz planes in strips of a shape and chunk, up to a factor. A
-// chunk of c planes costs its strip c + 4 planes (two beside its own, and as
-// much again to start). plane[n] is nearly n times one where the SM is full,
-// latency below. In a wave or two the fullest SM decides, and strips differ
-// (walls); many waves even out, but for the end of the last one.
-inline double strip_cost(int64_t nz, int64_t strips, int64_t chunk, int sms, const StripShapeCost& s)
+// Time of a step of that many strips of a shape and of chunk planes each, up to a
+// factor. A strip of c planes costs c + 4 planes (two beside its own, and as much
+// again to start). plane[n] is nearly n times one where the SM is full, latency
+// below. In a wave or two the fullest SM decides, and strips differ (walls); many
+// waves even out, but for the end of the last one.
+inline double strip_cost(int64_t strips, int64_t chunk, int sms, const StripShapeCost& s)
 {
-    const int64_t blocks = (strips * ((nz + chunk - 1) / chunk) + STRIP_WARPS - 1) / STRIP_WARPS;
+    const int64_t blocks = (strips + STRIP_WARPS - 1) / STRIP_WARPS;
     const double planes = (double)chunk + 4, waves = (double)blocks / ((double)sms * s.minb);
     if (waves <= 1) return planes * 1.15 * s.plane[(blocks + sms - 1) / sms];
     if (waves <= 2.5) return planes * s.plane[s.minb] * 1.15 * std::ceil(waves);
@@ -89,7 +89,7 @@ inline StripPlan strip_plan(int q, int storage, int variant, int nx, int ny, int
         const StripShapeCost s = strip_shape(q, storage, shape);
         const int64_t strips = strips_of(nx, ny, periodic_x, s.rows), planes = nz;
         auto take = [&](int64_t c) {
-            const double cost = strip_cost(planes, strips, c, sms, s);
+            const double cost = strip_cost(strips * ((planes + c - 1) / c), c, sms, s);
             if (least < 0 || cost < least) {
                 best = {shape, (int)c};
                 least = cost;
@@ -106,6 +106,43 @@ inline StripPlan strip_plan(int q, int storage, int variant, int nx, int ny, int
             c = (planes + n - 1) / n;
         }
     }
+    return best;
+}
+
+// Compact layout: how the strips of its tile columns (zchunk planes, `strips` strips
+// of them; storage and shape as above) and its node list share a step.
+//   planes: of a strip, a part of zchunk that divides it. Strips of whole columns
+//   leave small boxes to the latency of 24 planes: 160 x 288 x 58 at 29% fluid 59 us per
+//   step, 32 in parts (D3Q19 FP32). The list's blocks run beside the strips, so that
+//   waves even out; FP64 strips are their own bound.
+//   first: the strips are launched before the list and the list may start beside them.
+//   That pays where they fill the GPU at most once (128^3 at 40% 33 and 25 us) and the list's
+//   blocks are few, too: beside FP32 strips, which take nearly all shared memory, a
+//   gather finds little L1 (192^3 at 30%, f* = 0.5: 61 us with the list first, 81 so). The
+//   16-bit strips leave it its L1 (192^3 BF16 58 and 53 us).
+struct CompactPlan {
+    int planes;
+    bool first;
+};
+inline CompactPlan compact_plan(int q, int storage, int shape, int zchunk, int64_t strips, int64_t listed, int sms)
+{
+    const StripShapeCost s = strip_shape(q, storage, shape);
+    const double wave = (double)STRIP_WARPS * sms * s.minb;
+    CompactPlan best{zchunk, false};
+    double least = -1;
+    for (int n = 1; n <= zchunk / 4; ++n) {
+        if (zchunk % n != 0) continue;
+        const int64_t count = strips * n, planes = zchunk / n;
+        const double waves = (double)count / wave;
+        const double cost = waves <= 1 || storage == 0 ? strip_cost(count, planes, sms, s)
+                                                       : ((double)planes + 4) * s.plane[s.minb] * (waves + 0.4);
+        if (least < 0 || cost < least) {
+            best = {(int)planes, waves <= 1};
+            least = cost;
+        }
+    }
+    const int64_t resident = (int64_t)2 * 12 * 128 * sms;  // two waves of the list's threads (D3Q19)
+    best.first = best.first && (storage >= 2 || listed <= resident);
     return best;
 }
 

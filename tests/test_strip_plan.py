@@ -67,3 +67,32 @@ def test_fp32_boxes_take_the_faster_shape(plans):
              (27, (96, 256, 128), four), (19, (100, 300, 120), four), (19, (160, 160, 160), four), (27, (320, 320, 320), two)]
     got = plans([(q, 1, 0, *d, 1, 152) for q, d, _ in boxes])
     assert [rows for _, _, rows, _, _ in got] == [rows for _, _, rows in boxes]
+
+
+def test_compact_strips_are_cut_where_they_are_few(tmp_path):
+    """Strips of whole tile columns (24 or 32 planes) only where they fill the GPU; a
+    part always divides the column. The list waits for strips that fill it more than
+    once."""
+    (tmp_path / "c.cpp").write_text(r"""
+#include <cstdio>
+#include <initializer_list>
+#include "strip_plan.h"
+int main()
+{
+    for (int q : {19, 27})
+        for (int st = 0; st < 4; ++st)
+            for (int z : {24, 32})
+                for (long long n : {1ll, 100ll, 1000ll, 3000ll, 100000ll, 1ll << 30})
+                    for (long long l : {1000ll, 10000000ll}) {
+                        const lbm::CompactPlan p = lbm::compact_plan(q, st, 0, z, n, l, 152);
+                        std::printf("%d %d %lld %lld %d %d\n", st, z, n, l, p.planes, (int)p.first);
+                    }
+}
+""")
+    exe = str(tmp_path / "c")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-ftrapv", "-I", CSRC, str(tmp_path / "c.cpp"), "-o", exe])
+    for line in subprocess.check_output([exe], text=True).splitlines():
+        st, z, n, listed, part, first = map(int, line.split())
+        assert 4 <= part <= z and z % part == 0
+        assert part < z if n <= 100 else (n < 100000 or part == z), line
+        assert first == (1 if n <= 100 and (st >= 2 or listed == 1000) else 0) or 100 < n < 100000, line
