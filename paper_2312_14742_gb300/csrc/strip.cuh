@@ -17,6 +17,11 @@
 // around its strip gathers its nodes next to a wall, a few percent, into a list
 // and finishes 64 at a time, two per lane (bounce()), so that wall terms cost
 // one pass over 64 nodes and not one over every node of the strip.
+// Media crowded with walls pay for that list: 256^3 D3Q19 FP32 at 50% porosity takes 156
+// us with spheres of radius 6 and 168 with radius 3, where the tile kernels, which
+// carried wall terms for every node, took 155. (162 and 174 while nodes at solid
+// corners, where D3Q19 has no links, were listed too and the list was written word
+// by word; 138 instead of 134 at 90%, radius 8.)
 //
 // Records come by cp.async, each lane copying those it will read itself, one
 // plane ahead: no alignment rule besides the record's own, periodic images and
@@ -27,8 +32,8 @@
 // and more values along x.
 //
 // 256^3, spheres of radius 8 at 90% porosity, us per step by default, and of the
-// tile kernels before: D3Q19 FP32 136 (156), BF16 150 (183), D3Q27 FP32 147 (261), BF16
-// 206 (315); 128^3 D3Q19 FP64 702 (934). FP32 is bound by issue and the latency of
+// tile kernels before: D3Q19 FP32 134 (156), BF16 150 (183), D3Q27 FP32 144 (261), BF16
+// 206 (315); 128^3 D3Q19 FP64 687 (934). FP32 is bound by issue and the latency of
 // the 12 warps per SM of four-row strips, not by HBM (74 us for the state alone).
 // Blocks whose four warps met at a barrier per plane and formed 32 own columns each
 // took 10 to 23% more.
@@ -295,8 +300,12 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Place& pl, i
             const uint32_t bB = cvel(K, 0) == 1 ? iB.y : (cvel(K, 0) == 0 ? iB.z : iB.w);
             add(lanes_of(bA & bit ? v.v.x : E(0), bB & bit ? v.v.y : E(0)));
         }, Bn);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) s[f] = lanes_of(part[4 * eA + f], part[4 * eB + f]) + Bn[f];
+        const Rec<E> pA = read(reinterpret_cast<const unsigned char*>(part + 4 * eA)),
+                     pB = read(reinterpret_cast<const unsigned char*>(part + 4 * eB));
+        s[0] = lanes_of(pA.d, pB.d) + Bn[0];
+        s[1] = lanes_of(pA.ux, pB.ux) + Bn[1];
+        s[2] = lanes_of(pA.uy, pB.uy) + Bn[2];
+        s[3] = lanes_of(pA.uz, pB.uz) + Bn[3];
         L d, ux, uy, uz;
         node_state<Q, L>(s, d, ux, uy, uz);
         step_store<ST>(a.post, iA.x, d.v.x, ux.v.x, uy.v.x, uz.v.x, nullptr, a.seed);
@@ -369,9 +378,16 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Place& pl, i
         if (__any_sync(0xffffffffu, hist != 0u)) {
             // solid bits of the columns left and right, and of all three together
             const uint32_t hl = __shfl_sync(0xffffffffu, hist, pl.left), hr = __shfl_sync(0xffffffffu, hist, pl.right);
-            uint32_t n3 = hist | hl | hr;
-            n3 |= n3 >> B | n3 >> (2 * B);
-            const uint32_t lst = store & (n3 | n3 << 1 | n3 >> 1);  // rows next to a wall
+            // rows next to a wall; D3Q19 has no links to the corners
+            uint32_t lst;
+            if constexpr (Q == 19) {
+                const uint32_t side = hl | hr, own = hist | hist >> B | hist >> (2 * B), rows = own | side >> B;
+                lst = store & (rows | rows << 1 | rows >> 1 | side | side >> (2 * B));
+            } else {
+                uint32_t n3 = hist | hl | hr;
+                n3 |= n3 >> B | n3 >> (2 * B);
+                lst = store & (n3 | n3 << 1 | n3 >> 1);
+            }
             store &= ~lst;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -379,13 +395,14 @@ __device__ __forceinline__ void strip_step(const StepArgs& a, const Place& pl, i
                 const uint32_t m = __ballot_sync(0xffffffffu, mineq);
                 if (mineq) {
                     const int e = waiting + __popc(m & ((1u << lane) - 1u));
-                    E* q = part + 4 * e;
+                    E q[4];
 #pragma unroll
                     for (int f = 0; f < 4; ++f) q[f] = r < NP ? s[r % NP][f].v.x : s[r % NP][f].v.y;
+                    Storage<ST>::store(part, (uint32_t)e, q[0], q[1], q[2], q[3], nullptr);
                     const unsigned char* rec = planes.cell(slot == 0 ? C::NSTAGE - 1 : slot - 1, r);
 #pragma unroll
-                    for (int k = 0; k < REC / 8; ++k)
-                        reinterpret_cast<uint2*>(raw + e * REC)[k] = reinterpret_cast<const uint2*>(rec)[k];
+                    for (int k = 0; k < REC / 16; ++k)
+                        reinterpret_cast<uint4*>(raw + e * REC)[k] = reinterpret_cast<const uint4*>(rec)[k];
                     ids[e] = make_uint4(zoff + xy + (uint32_t)(r * a.nx), hl >> r, hist >> r, hr >> r);
                 }
                 waiting += __popc(m);
